@@ -40,6 +40,13 @@ bool use_c64p4_pf(const Prm& pr) {
   return pr.C == 64 && pr.P == 4 && pr.variant == AWSRC_VARIANT_PF;
 }
 
+// The mma.sync search: tiles of whole k-steps, two or four atoms. (For C = 4, 8
+// half or more of a k-step would be padding; C = 256 and P up to 8 do not fit
+// its registers: those shapes keep the scalar search.)
+bool use_mma(const Prm& pr) {
+  return pr.C >= 16 && pr.C <= 128 && (pr.P == 2 || pr.P == 4) && !use_c64p4(pr) && !use_c64p4_pf(pr);
+}
+
 bool aligned(const void* p, uintptr_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
 uintptr_t elt_bytes(int32_t dtype) { return dtype == AWSRC_DTYPE_BF16 ? 2 : 4; }
 
@@ -76,12 +83,14 @@ struct EncodeLayout {
   int nsplit;
   bool spec;     // U, C = 64, P = 4: tcgen05 search
   bool spec_pf;  // P_F, C = 64, P = 4: tcgen05 search
+  bool mma;      // mma.sync search
 };
 
 EncodeLayout encode_layout(const Prm& pr, int32_t n_mod, const awsrc_module* mods, int64_t T) {
   EncodeLayout L{};
   L.spec = use_c64p4(pr);
   L.spec_pf = use_c64p4_pf(pr);
+  L.mma = use_mma(pr);
   const GenShape gs = gen_shape(pr);
   int64_t base_blocks = 0, ncb = 0;
   for (int m = 0; m < n_mod; ++m) {
@@ -89,9 +98,11 @@ EncodeLayout encode_layout(const Prm& pr, int32_t n_mod, const awsrc_module* mod
     ncb += n_cb;
     if (L.spec || L.spec_pf) base_blocks += n_cb * ((mods[m].rows + search_c64p4_rows() - 1) / search_c64p4_rows());
   }
-  if (!(L.spec || L.spec_pf)) base_blocks = (T + gs.tiles - 1) / gs.tiles;
+  const int64_t tiles = L.mma ? search_mma_tiles() : gs.tiles;
+  if (!(L.spec || L.spec_pf)) base_blocks = (T + tiles - 1) / tiles;
   const int64_t units = L.spec ? pr.S_pad / search_c64p4_chunk()
                        : L.spec_pf ? pr.S_pad / search_pf_c64p4_chunk()
+                       : L.mma     ? (pr.S + 7) / 8  // groups of eight seeds
                                    : (pr.S + gs.lanes - 1) / gs.lanes;
   int64_t ns = (kTargetBlocks + base_blocks - 1) / base_blocks;
   ns = std::max<int64_t>(1, std::min<int64_t>(ns, units));
@@ -100,10 +111,11 @@ EncodeLayout encode_layout(const Prm& pr, int32_t n_mod, const awsrc_module* mod
   L.masks = off;
   off += align_up((size_t)pr.S_pad * pr.P * pr.W * 8, 256);
   L.gram = off;  // read by the generic U search
-  if (pr.variant == AWSRC_VARIANT_U && !L.spec)
+  if (pr.variant == AWSRC_VARIANT_U && !L.spec && !L.mma)
     off += align_up((size_t)ncb * pr.S_pad * gram_stride(pr.P) * 4, 256);
   L.pairs = off;
-  if (L.spec) off += align_up((size_t)ncb * (pr.S_pad / 2) * pair_stride(pr.P) * 8, 256);
+  if (L.spec || (L.mma && pr.variant == AWSRC_VARIANT_U))
+    off += align_up((size_t)ncb * (pr.S_pad / 2) * pair_stride(pr.P) * 8, 256);
   L.mexp = off;
   if (L.spec || L.spec_pf) off += align_up(search_c64p4_table_bytes(pr.S_pad), 256);
   L.ptab = off;
@@ -422,9 +434,10 @@ awsrc_status awsrc_encode_tiles(const awsrc_params* prm, int32_t n_mod, const aw
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   uint32_t* status = reinterpret_cast<uint32_t*>(ws);
   uint64_t* masks = reinterpret_cast<uint64_t*>(ws + lay.masks);
-  float* gram = lay.spec ? nullptr : reinterpret_cast<float*>(ws + lay.gram);
+  const bool paired = lay.spec || lay.mma;
+  float* gram = paired ? nullptr : reinterpret_cast<float*>(ws + lay.gram);
   awsrc_candidate* pcands = lay.nsplit > 1 ? reinterpret_cast<awsrc_candidate*>(ws + lay.pcands) : out;
-  float2* pairs = lay.spec ? reinterpret_cast<float2*>(ws + lay.pairs) : nullptr;
+  float2* pairs = paired ? reinterpret_cast<float2*>(ws + lay.pairs) : nullptr;
   void* mexp = ws + lay.mexp;
   cudaError_t e = cudaMemsetAsync(status, 0, sizeof(uint32_t), st);
   if (e != cudaSuccess) return cuda_fail(e, "encode: clear status");
@@ -461,9 +474,10 @@ awsrc_status awsrc_encode_tiles(const awsrc_params* prm, int32_t n_mod, const aw
       tile_off += d.rows * d.n_cb;
       gram_off += d.n_cb * pr.S_pad;
     }
-    if (!spec) {  // the generic search takes runs of consecutive tiles
+    if (!spec) {  // the other searches take runs of consecutive tiles
       const int64_t tiles = tile_off - ld.m[0].tile_off;
-      blocks = (tiles + gs.tiles - 1) / gs.tiles * lay.nsplit;
+      const int64_t run = lay.mma ? search_mma_tiles() : gs.tiles;
+      blocks = (tiles + run - 1) / run * lay.nsplit;
     }
     if (pr.variant == AWSRC_VARIANT_U && (e = launch_gram_u(pr, ld, masks, gram, pairs, st)) != cudaSuccess)
       return cuda_fail(e, "encode: gram");
@@ -471,6 +485,9 @@ awsrc_status awsrc_encode_tiles(const awsrc_params* prm, int32_t n_mod, const aw
       return cuda_fail(e, "encode: timing event");
     if (lay.spec) e = launch_search_c64p4(pr, ld, mexp, pairs, masks, blocks, pcands, status, st);
     else if (lay.spec_pf) e = launch_search_pf_c64p4(pr, ld, mexp, ptab, masks, blocks, pcands, status, st);
+    else if (lay.mma)
+      e = pr.variant == AWSRC_VARIANT_U ? launch_search_mma_u(pr, ld, masks, pairs, blocks, pcands, st)
+                                        : launch_search_mma_pf(pr, ld, masks, blocks, pcands, st);
     else e = launch_search_generic(pr, ld, masks, gram, blocks, pcands, st);
     if (e != cudaSuccess) return cuda_fail(e, "encode: search");
     if (g0 + kMaxModsPerLaunch >= n_mod && g_ev_after && (e = cudaEventRecord(g_ev_after, st)) != cudaSuccess)

@@ -1,5 +1,7 @@
 // encode.cu — the seed search of Sec. 3.2 for any supported (C, P) and both
-// variants, and the U Gram tables every U search reads:
+// variants (the tensor-core searches take C = 64, P = 4 and, for P in {2, 4}, C = 16
+// to 128; this scalar one serves the rest), and the U Gram tables every U search
+// reads:
 //
 //  gram_u      U only. The activation diagonal is shared by all rows of a module
 //              (Sec. 3.2), so the Gram matrix B_s^T D B_s of Eq. 3 and its LDL^T

@@ -42,6 +42,14 @@ GenShape gen_shape(const Prm& pr);
 cudaError_t launch_search_generic(const Prm& pr, const LaunchDesc& ld, const uint64_t* masks,
                                   const float* gram, int64_t n_blocks, awsrc_candidate* cands,
                                   cudaStream_t st);
+// search_mma_u.cu, search_mma_pf.cu: the search for C in {16, 32, 64, 128} and
+// P in {2, 4} (search_mma.cuh) in items of search_mma_tiles() consecutive tiles
+// and one seed split; same candidate output. `pairs`: the paired Gram table.
+int search_mma_tiles();
+cudaError_t launch_search_mma_u(const Prm& pr, const LaunchDesc& ld, const uint64_t* masks, const float2* pairs,
+                                int64_t n_items, awsrc_candidate* cands, cudaStream_t st);
+cudaError_t launch_search_mma_pf(const Prm& pr, const LaunchDesc& ld, const uint64_t* masks, int64_t n_items,
+                                 awsrc_candidate* cands, cudaStream_t st);
 // search_c64p4.cu
 // FP16 table of the +-1 atoms in MMA operand order, then the tcgen05 search.
 size_t search_c64p4_table_bytes(int S_pad);
