@@ -531,6 +531,7 @@ static awsrc_status select_plan(const Prm& pr, int32_t n_mod, const awsrc_module
   for (int r = 0; r < n_rates; ++r)
     if (!(rates[r] >= 0.0) || !std::isfinite(rates[r])) return AWSRC_ERR_INVALID_ARG;
   kcap->clear();
+  int key_bits;  // module, gain field and tile: the range of calls the ABI takes
   if (pr.variant == AWSRC_VARIANT_U) {
     const int64_t B = (int64_t)std::floor(rates[0] * (double)N / 8.0);
     if (B < sp->h) return AWSRC_ERR_BUDGET;
@@ -544,9 +545,7 @@ static awsrc_status select_plan(const Prm& pr, int32_t n_mod, const awsrc_module
       cap += k;
     }
     sp->cap_records = cap;
-    sp->tile_bits_local = ceil_log2_host((uint64_t)maxTm);
-    sp->mod_shift = 31 + sp->tile_bits_local;
-    sp->key_bits = sp->mod_shift + ceil_log2_host((uint64_t)n_mod);
+    key_bits = 31 + ceil_log2_host((uint64_t)maxTm) + ceil_log2_host((uint64_t)n_mod);
   } else {
     int64_t cap = 0;
     for (int r = 0; r < n_rates; ++r) {
@@ -557,12 +556,9 @@ static awsrc_status select_plan(const Prm& pr, int32_t n_mod, const awsrc_module
       cap = std::max(cap, k);
     }
     sp->cap_records = cap;
-    sp->tile_bits_local = ceil_log2_host((uint64_t)T);
-    sp->mod_shift = 0;
-    sp->key_bits = 31 + sp->tile_bits_local;
+    key_bits = 31 + ceil_log2_host((uint64_t)T);
   }
-  if (sp->key_bits > 64) return AWSRC_ERR_UNSUPPORTED;
-  sp->nblocks = (T + 2047) / 2048;
+  if (key_bits > 64) return AWSRC_ERR_UNSUPPORTED;
   return AWSRC_OK;
 }
 
@@ -589,8 +585,8 @@ awsrc_status awsrc_select_workspace_bytes(const awsrc_params* prm, int32_t n_mod
   if ((s = check_modules(pr, n_mod, mods, false, &T)) != AWSRC_OK) return s;
   SelectPlan sp{};
   sp.T = T;
-  sp.nblocks = (T + 2047) / 2048;
-  *bytes = select_ws_bytes(sp);
+  sp.n_mod = n_mod;
+  *bytes = select_ws_bytes(pr, sp);
   return AWSRC_OK;
 }
 
@@ -608,14 +604,10 @@ awsrc_status awsrc_select_records(const awsrc_params* prm, int32_t n_mod, const 
   if (!cands || !stream_out || !d_counts || !d_bytes) return AWSRC_ERR_INVALID_ARG;
   if (!aligned(cands, 4) || !aligned(d_counts, 8) || !aligned(d_bytes, 8)) return AWSRC_ERR_INVALID_ARG;
   if (stream_capacity < (size_t)(sp.h + sp.cap_records * sp.L)) return AWSRC_ERR_CAPACITY;
-  if (!workspace || workspace_bytes < select_ws_bytes(sp)) return AWSRC_ERR_WORKSPACE;
+  if (!workspace || workspace_bytes < select_ws_bytes(pr, sp)) return AWSRC_ERR_WORKSPACE;
   if (!aligned(workspace, 256)) return AWSRC_ERR_INVALID_ARG;
-  std::vector<int64_t> mt(n_mod);
-  for (int m = 0; m < n_mod; ++m) mt[m] = to[m + 1] - to[m];
-  const cudaError_t e = cudaMemsetAsync(workspace, 0, sizeof(uint32_t), (cudaStream_t)stream);
-  if (e != cudaSuccess) return cuda_fail(e, "select: clear status");
-  return select_run(pr, sp, to.data(), mt.data(), kc.data(), cands, stream_out, d_counts, d_bytes,
-                    workspace, workspace_bytes, (cudaStream_t)stream);
+  return select_run(pr, sp, to.data(), kc.data(), cands, stream_out, d_counts, d_bytes, workspace, workspace_bytes,
+                    (cudaStream_t)stream);
 }
 
 // ------------------------------------------------------------------ decode --

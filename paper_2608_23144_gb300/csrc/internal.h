@@ -77,15 +77,14 @@ cudaError_t launch_search_pf_c64p4(const Prm& pr, const LaunchDesc& ld, const vo
 struct SelectPlan {
   int n_mod, n_rates;
   int64_t T, L, h;
-  int key_bits, tile_bits_local, mod_shift;
   int64_t cap_records;      // upper bound on records written
-  int64_t nblocks;          // radix blocks
 };
+// Clears the workspace's status word, then selects and serialises.
 awsrc_status select_run(const Prm& pr, const SelectPlan& sp, const int64_t* tile_off,
-                        const int64_t* mod_tiles, const int64_t* kcap /* U: per module; PF: per rate */,
+                        const int64_t* kcap /* U: per module; PF: per rate */,
                         const awsrc_candidate* cands, uint8_t* stream_out, int64_t* d_counts,
                         int64_t* d_bytes, void* ws, size_t ws_bytes, cudaStream_t st);
-size_t select_ws_bytes(const SelectPlan& sp);
+size_t select_ws_bytes(const Prm& pr, const SelectPlan& sp);
 
 // decode.cu
 struct DecodeMod {

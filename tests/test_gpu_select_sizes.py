@@ -20,6 +20,9 @@ CASES = [
     (dict(C=4, P=2, b=3, S=9, variant=U), [(1, 4), (2048, 4), (2049, 8), (4095, 4)], [4.0], 1, 0),
     (dict(C=4, P=2, b=4, S=16, variant=PF), [(300001, 4), (1, 4), (512, 1024), (700000, 8)], [2.5, 8.0, 12.0], 7, 0),
     (dict(C=4, P=2, b=4, S=16, variant=U), [(300001, 4), (1, 4), (512, 1024), (700000, 8)], [9.0], 0, 3),
+    # more tiles than a block compacts in one turn; four passes (every gain kept)
+    (dict(C=4, P=4, b=4, S=4096, variant=PF), [(1 << 20, 16), (5001, 4), (64, 1024)], [1.3, 14.0], 5, 0),
+    (dict(C=8, P=8, b=8, S=4096, scale_mode=1, b_e=16, variant=U), [(1 << 21, 8), ((1 << 21) + 77, 8)], [4.0], 0, 0),
 ]
 
 
