@@ -435,8 +435,8 @@ awsrc_status awsrc_decode_apply_inplace_noalloc(const awsrc_params* prm, int32_t
  *   aligned; y is M x rows): W0_ij = fl(q_ij * s_eff) from the packed backbone
  *   (awsrc_rtn_quantize's outputs; binary16 scales or SDQ), r_ij =
  *   fl(fl(k_j * C^-1/2) * scale) on the tiles the sidecar names (none when
- *   `sidecar` is NULL), both accumulated in binary32 with fma (the residual
- *   terms in their own sums). The result equals the double-precision product
+ *   `sidecar` is NULL), both accumulated in binary32 (the residual terms in
+ *   their own sums; x enters the sums unrounded). The result equals the double-precision product
  *   sum_j (W0_ij + r_ij) x_j, r_ij = k_j C^-1/2 scale, within
  *   (cols / min(C, 32) + 32) * 2^-24 * sum_j (|W0_ij x_j| + |r_ij x_j|).
  *   The module needs cols % 128 == 0.

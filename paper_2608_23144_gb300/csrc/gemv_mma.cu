@@ -1,0 +1,352 @@
+// gemv_mma.cu — the packed product y[m] = (W0 + r_hat) x[m], m < M <= 8, on the
+// tensor cores, for the codes of the code tables (P = 4, b <= 5, C in {16, 32, 64})
+// with power-of-two scales, or no sidecar; gemv.cu serves the rest.
+//
+// One weight matrix against up to eight vectors: every weight is read once (0.68
+// bytes with its scale and sidecar), so on the FP32 pipes the unpacking, one FMA
+// per weight and vector and the x operands' shared-memory reads decide (24 M warp
+// instructions for a 3B layer and one vector; eight vectors took ten times the
+// time). With mma.sync m16n8k16 the eight vectors are the N columns of one
+// instruction and cost the same as one:
+//  * A: 16 rows of 4-bit codes as exact BF16 integers, from the code words by one
+//    mask-and-xor into the mantissa of 128 + u and one packed subtraction;
+//  * B: x as x = hi + mid + lo, three BF16 numbers whose sum is x exactly (8 + 8 + 8
+//    significand bits by truncation), so a product loses nothing that binary32
+//    holds; the chain of the hi parts and that of the mid and lo parts have their own
+//    binary32 accumulators, over one group of 128 inputs each. A group's sum is
+//    multiplied by its scale and added with binary32 FMAs, as before.
+//  * The residual: k_j c 2^e is exact in BF16 (|k_j| <= 64), so recorded tiles are a
+//    second A operand against the same B (rows without a record: zeros), with its own
+//    accumulators; column runs without any record in the 16 rows are skipped.
+// The order of the inputs along K is free: in each run of 32 inputs thread (g, q) =
+// (lane / 4, lane % 4) takes inputs 8q .. 8q + 7, one code word of rows g and g + 8, one
+// nibble-table window, two float4 of vector g.
+//
+// A warp takes 16 rows and a slice of the columns; slices of a row tile sit in one
+// block and are summed through shared memory in a fixed order, so a product's bits do
+// not depend on what shares its launch.
+//
+// One 3B-shaped layer (77 M weights, 0.162 bits/weight of records, SDQ scales, eight
+// vectors, one batched launch): 263 -> 69 us on the device, 308 -> 76 us a call. Its
+// relative error against 64 bits is 9.6e-8 where the FP32 pipes' sums had 1.4e-7.
+// Bound by issue (46% of slots): 370 instructions per 16 rows and 128 inputs for the
+// backbone (half of them the split of x) and up to 380 for the residual.
+#include "codetab.cuh"
+#include "internal.h"
+
+namespace awsrc {
+
+namespace {
+
+constexpr int kWarps = 8;
+
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+      "{%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Upper halves of two binary32 numbers as a BF16 pair (a in the low half).
+__device__ __forceinline__ uint32_t upper_pair(float a, float b) {
+  return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632);
+}
+__device__ __forceinline__ float upper(float a) { return __uint_as_float(__float_as_uint(a) & 0xffff0000u); }
+
+// B operand of a run of 32 inputs (two k-steps): pairs (x_i, x_{i+4}), i < 4, of
+// this thread's eight inputs, split into three BF16 parts.
+struct BRun {
+  uint32_t hi[4], mid[4], lo[4];
+};
+
+// Returns whether one of the eight inputs is an infinity or NaN.
+__device__ __forceinline__ bool split_run(const float4& xa, const float4& xb, BRun& b) {
+  const float a[4] = {xa.x, xa.y, xa.z, xa.w}, c[4] = {xb.x, xb.y, xb.z, xb.w};
+  float2 r[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    b.hi[i] = upper_pair(a[i], c[i]);
+    r[i] = __fadd2_rn(make_float2(a[i], c[i]), make_float2(-upper(a[i]), -upper(c[i])));
+    b.mid[i] = upper_pair(r[i].x, r[i].y);
+    const float2 s = __fadd2_rn(r[i], make_float2(-upper(r[i].x), -upper(r[i].y)));
+    b.lo[i] = upper_pair(s.x, s.y);
+  }
+  // an infinity or NaN leaves a NaN remainder: keep it in hi alone, so that it
+  // enters the products once, as itself
+  const float2 t = __fadd2_rn(__fadd2_rn(r[0], r[1]), __fadd2_rn(r[2], r[3]));
+  const float n = __fadd_rn(t.x, t.y);
+  if (n != n) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      b.hi[i] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a[i])) |
+                ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(c[i])) << 16);
+      b.mid[i] = b.lo[i] = 0u;
+    }
+    return true;
+  }
+  return false;
+}
+
+// Codes i and i + 4 of a code word as a BF16 pair: 128 + u (u = code + 8) in the
+// mantissa, minus 136.
+__device__ __forceinline__ uint32_t code_pair(uint32_t w, int i) {
+  const uint32_t v = ((w >> (4 * i)) & 0x000F000Fu) ^ 0x43084308u;
+  uint32_t r;
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(0x43084308u));
+  return r;
+}
+
+// acc += A B over a run: A as pairs (element i, element i + 4) of rows g and g + 8.
+__device__ __forceinline__ void mma_run(float (&h)[4], float (&ml)[4], const uint32_t (&r0)[4],
+                                        const uint32_t (&r1)[4], const BRun& b) {
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const uint32_t a[4] = {r0[2 * s], r1[2 * s], r0[2 * s + 1], r1[2 * s + 1]};
+    mma_bf16(ml, a, b.lo[2 * s], b.lo[2 * s + 1]);
+    mma_bf16(ml, a, b.mid[2 * s], b.mid[2 * s + 1]);
+    mma_bf16(h, a, b.hi[2 * s], b.hi[2 * s + 1]);
+  }
+}
+
+// What a thread needs of a recorded tile of its row: the record's byte tables as
+// k_j + 64, and 2^(e - S) in both halves of a BF16 pair (k_j 2^(e - S) is k_j c 2^e
+// for C = 64 and 16, k_j 2^e / 4 for C = 32; 2^(e - S) may be a subnormal BF16).
+struct TileRec {
+  KTab kt;
+  uint32_t sc;
+  uint32_t seed;
+};
+
+template <int LC>
+__device__ __forceinline__ TileRec tile_rec(const GemvArgs& a, unsigned long long e) {
+  TileRec t{{0u, 0u, 0u, 0u}, 0u, 0u};
+  if (e == 0ull) return t;
+  const uint4 slot = __ldg(a.slots + ((int64_t)(e >> 32) - 1));
+  // k_tables() gives k + 128 as bytes of 64 .. 192
+  const KTab k = k_tables(slot);
+  t.kt = {k.t0 - 0x40404040u, k.t1 - 0x40404040u, k.u0 - 0x40404040u, k.u1 - 0x40404040u};
+  constexpr int S = LC == 6 ? 3 : 2;
+  const int f = (int)(int16_t)(uint16_t)(e & 0xFFFFull) - S;
+  const uint32_t sb = f >= -126 ? (uint32_t)(f + 127) << 7 : 1u << (f + 133);
+  t.sc = sb * 0x00010001u;
+  t.seed = (uint32_t)(e >> 16) & 0xFFFFu;
+  return t;
+}
+
+// The residual of this thread's eight inputs (window nb of the seed's nibble
+// table) as pairs (i, i + 4): the byte k + 64 completes 128 + (k + 64) in the
+// mantissa (128 carries into the next binade, which is right), minus 192, times
+// the scale, all exact; zeros where sc is 0 (no record).
+__device__ __forceinline__ void residual_pairs(const TileRec& t, const uint4& nb, uint32_t (&r)[4]) {
+  const uint32_t s0 = nb.x & 0xFFFFu, s1 = nb.x >> 16;
+  const uint32_t a0 = __byte_perm(t.kt.t0, t.kt.t1, s0), b0 = __byte_perm(t.kt.u0, t.kt.u1, s0);
+  const uint32_t a1 = __byte_perm(t.kt.t0, t.kt.t1, s1), b1 = __byte_perm(t.kt.u0, t.kt.u1, s1);
+  const uint32_t k0 = (a0 & ~nb.y) | (b0 & nb.y), k1 = (a1 & ~nb.z) | (b1 & nb.z);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t v = (__byte_perm(k0, k1, 0x0400u + 0x0101u * i) & 0x00FF00FFu) | 0x43004300u;
+    uint32_t d;
+    asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(v), "r"(0x43404340u));
+    asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r[i]) : "r"(d), "r"(t.sc));
+  }
+}
+
+template <int LC>
+__global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const __grid_constant__ GemvArgs a, int M) {
+  __shared__ float4 part[kWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+  int ti = 0;
+  for (int i = 1; i < a.n_task; ++i)
+    if ((int)blockIdx.x >= a.t[i].block0) ti = i;
+  const GemvTask& tk = a.t[ti];
+  const int ks = tk.slices, slice = warp & (ks - 1), per = kWarps / ks;  // slices: a power of two up to kWarps
+  const int64_t row0 = ((int64_t)(blockIdx.x - tk.block0) * per + warp / ks) * 16;
+  const int gpr = (int)(tk.cols >> 7);
+  const int g0 = gpr * slice / ks, g1 = row0 < tk.rows ? gpr * (slice + 1) / ks : g0;
+  int64_t row[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) row[r] = min(row0 + g + 8 * r, tk.rows - 1);  // rows past the end repeat the last one
+  const uint32_t* cp[2];
+  const unsigned long long* mp[2];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    cp[r] = reinterpret_cast<const uint32_t*>(tk.codes) + row[r] * (tk.cols >> 3) + q;
+    mp[r] = a.map ? a.map + tk.tile_off + row[r] * (tk.cols >> LC) : nullptr;
+  }
+  const bool live = g < M;  // vector g
+  const float* xp = tk.x + (live ? (int64_t)g * tk.cols : 0) + 8 * q;
+  auto scale = [&](int r, int gr) {
+    const int64_t gid = row[r] * gpr + gr;
+    if (tk.sdq) {
+      const float2 ms = __ldg(reinterpret_cast<const float2*>(tk.sdq_consts) + (gid >> 8));
+      return __fadd_rn(ms.x, __fmul_rn((float)__ldg(tk.sdq_codes + gid), ms.y));
+    }
+    return __half2float(__ushort_as_half(__ldg(tk.scales + gid)));
+  };
+  // A group's code words, scales and (a tile per 2^LC inputs) map entries, one group ahead
+  constexpr int NT = LC >= 5 ? 128 >> LC : 4;  // entries per group, row and thread
+  uint32_t w[2][4];
+  unsigned long long e[2][NT];
+  float s[2];
+  auto load = [&](int gr) {
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) w[r][j] = __ldg(cp[r] + 16 * gr + 4 * j);
+      s[r] = scale(r, gr);
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+        e[r][t] = mp[r] ? __ldg(mp[r] + (LC >= 5 ? NT * gr + t : 8 * gr + 2 * t + (q >> 1))) : 0ull;
+    }
+  };
+  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, racc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  if (g0 < g1) load(g0);
+  for (int gr = g0; gr < g1; ++gr) {
+    uint32_t wc[2][4];
+    unsigned long long ec[2][NT];
+    const float sc[2] = {s[0], s[1]};
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) wc[r][j] = w[r][j];
+#pragma unroll
+      for (int t = 0; t < NT; ++t) ec[r][t] = e[r][t];
+    }
+    if (gr + 1 < g1) load(gr + 1);
+    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    float rh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    TileRec tr[2];
+    bool any = false;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float4 xa = make_float4(0.0f, 0.0f, 0.0f, 0.0f), xb = xa;
+      if (live) {
+        xa = __ldg(reinterpret_cast<const float4*>(xp + 128 * gr + 32 * j));
+        xb = __ldg(reinterpret_cast<const float4*>(xp + 128 * gr + 32 * j + 4));
+      }
+      const int t = LC == 6 ? j >> 1 : j;
+      if (LC != 6 || (j & 1) == 0) {  // a new tile
+        any = mp[0] && __any_sync(0xffffffffu, (ec[0][t] | ec[1][t]) != 0ull);
+        if (any) {
+          tr[0] = tile_rec<LC>(a, ec[0][t]);
+          tr[1] = tile_rec<LC>(a, ec[1][t]);
+        }
+      }
+      uint4 nb[2];
+      if (any) {
+        const int win = ((32 * j + 8 * q) & ((1 << LC) - 1)) >> 3;
+#pragma unroll
+        for (int r = 0; r < 2; ++r) nb[r] = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + win);
+      }
+      BRun b;
+      const bool bad = split_run(xa, xb, b);
+      uint32_t c0[4], c1[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        c0[i] = code_pair(wc[0][j], i);
+        c1[i] = code_pair(wc[1][j], i);
+      }
+      mma_run(h, ml, c0, c1, b);
+      if (any) {
+        residual_pairs(tr[0], nb[0], c0);
+        residual_pairs(tr[1], nb[1], c1);
+        if (!__any_sync(0xffffffffu, bad)) {
+          mma_run(rh, rml, c0, c1, b);
+        } else {
+          // a row without a record here must not meet 0 * infinity: the inputs of
+          // lanes with one go apart and count for recorded rows only
+          float th[4] = {0.0f, 0.0f, 0.0f, 0.0f}, tm[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+          BRun fin;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            fin.hi[i] = bad ? 0u : b.hi[i];
+            fin.mid[i] = bad ? 0u : b.mid[i];
+            fin.lo[i] = bad ? 0u : b.lo[i];
+            b.hi[i] = bad ? b.hi[i] : 0u;
+            b.mid[i] = b.lo[i] = 0u;
+          }
+          mma_run(rh, rml, c0, c1, fin);
+          mma_run(th, tm, c0, c1, b);
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const unsigned has = __ballot_sync(0xffffffffu, ec[r][t] != 0ull) >> (lane & 28) & 15u;
+            if (has) {
+              racc[2 * r] = __fadd_rn(racc[2 * r], __fadd_rn(th[2 * r], tm[2 * r]));
+              racc[2 * r + 1] = __fadd_rn(racc[2 * r + 1], __fadd_rn(th[2 * r + 1], tm[2 * r + 1]));
+            }
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      // an all-zero group (scale 0) adds nothing, whatever x holds
+      const float sr = sc[i >> 1];
+      if (sr != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sr, acc[i]);
+      racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
+    }
+  }
+  // c = 2^-(LC/2) is folded into the residual for C = 64 and 16; C = 32 had 1/4
+  const float cf = LC == 5 ? __fmul_rn(4.0f, pr.c) : 1.0f;
+  float v[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __fmaf_rn(racc[i], cf, acc[i]);
+  if (ks > 1) {
+    part[warp][lane] = make_float4(v[0], v[1], v[2], v[3]);
+    __syncthreads();
+    if (slice == 0) {
+      for (int i = 1; i < ks; ++i) {
+        const float4 p = part[warp + i][lane];
+        v[0] = __fadd_rn(v[0], p.x);
+        v[1] = __fadd_rn(v[1], p.y);
+        v[2] = __fadd_rn(v[2], p.z);
+        v[3] = __fadd_rn(v[3], p.w);
+      }
+    }
+  }
+  if (slice == 0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t r = row0 + g + 8 * (i >> 1);
+      const int m = 2 * q + (i & 1);
+      if (r < tk.rows && m < M) tk.y[(int64_t)m * tk.rows + r] = v[i];
+    }
+  }
+}
+
+}  // namespace
+
+// From three vectors on: the layer of the figures above takes 66 us here whatever
+// M is, against 30, 47, 125 and 263 us for M = 1, 2, 3 and 8 on the FP32 pipes.
+bool gemv_mma(const Prm& pr, const GemvArgs& a, int M) {
+  const bool c = pr.C == 16 || pr.C == 32 || pr.C == 64;
+  return M >= 3 && c && (!a.map || (a.nib && pr.scale_mode == AWSRC_SCALE_POW2));
+}
+
+cudaError_t launch_gemv_mma(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st) {
+  GemvArgs b = a;
+  int64_t blocks = 0;
+  for (int i = 0; i < b.n_task; ++i) {
+    GemvTask& t = b.t[i];
+    // slices of about eight groups: the shape alone decides, so that a product's
+    // sums are the same in every batch
+    const int64_t gpr = t.cols >> 7;
+    t.slices = 1;
+    while (t.slices < kWarps && gpr > 8 * t.slices) t.slices <<= 1;
+    const int64_t per = 16 * (kWarps / t.slices);
+    t.block0 = (int)blocks;
+    blocks += (t.rows + per - 1) / per;
+  }
+  if (blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
+  const dim3 grid((unsigned)blocks), block(32 * kWarps);
+  switch (pr.C) {
+    case 16: gemv_mma_kernel<4><<<grid, block, 0, st>>>(pr, b, M); break;
+    case 32: gemv_mma_kernel<5><<<grid, block, 0, st>>>(pr, b, M); break;
+    case 64: gemv_mma_kernel<6><<<grid, block, 0, st>>>(pr, b, M); break;
+    default: return cudaErrorInvalidValue;
+  }
+  note_launches(1);
+  return cudaGetLastError();
+}
+
+}  // namespace awsrc

@@ -113,7 +113,8 @@ bool decode_clears_status(const Prm& pr, int mode);
 // prepared sidecar, one launch for the tasks whose x fits in shared memory.
 struct GemvTask {
   int64_t rows, cols, tile_off;  // tile_off: the module's first global tile
-  int32_t sdq, block0;           // block0: the task's first block (set by launch_gemv)
+  int32_t sdq, block0;           // block0: the task's first block (set by the launch)
+  int32_t slices, pad_;          // gemv_mma.cu: column slices per row tile (set by the launch)
   const uint16_t* codes;         // 4 codes per uint16, element 2i in the low nibble of byte i
   const uint16_t* scales;        // binary16 per group (sdq == 0)
   const int8_t* sdq_codes;       // per group (sdq)
@@ -133,6 +134,9 @@ struct GemvArgs {
 // Whether the GEMV walks recorded tiles with the decoder's code tables.
 bool gemv_tables(const Prm& pr);
 cudaError_t launch_gemv(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st);
+// gemv_mma.cu: the same products on the tensor cores, where gemv_mma() says so.
+bool gemv_mma(const Prm& pr, const GemvArgs& a, int M);
+cudaError_t launch_gemv_mma(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st);
 
 // backbone.cu: RTN-INT4 groups of rtn_group() inputs, SDQ blocks of sdq_block() groups.
 int rtn_group();
