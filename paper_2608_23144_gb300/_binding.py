@@ -11,6 +11,7 @@ from __future__ import annotations
 
 import ctypes as ct
 import os
+import struct
 from typing import Dict, List, Optional, Sequence
 
 import numpy as np
@@ -239,6 +240,164 @@ def module_array(modules: Sequence[Dict[str, object]], decoder: bool = False):
     return arr
 
 
+# The calls below marshal many small tensors (a layer's packed product names 40),
+# and the checks above, one by one with their messages, cost more host time than
+# the kernels run (61 us for that product against 30 us on the device). So each
+# call first takes its arguments through one pass that tests the same conditions
+# without building anything and packs the C structs directly; when any condition
+# fails, or anything unusual is met, it returns None and the checked path above
+# decides (and raises what it always raised).
+_WEIGHT_DTYPES = {torch.float32: DTYPE_F32, torch.bfloat16: DTYPE_BF16}
+_MODULE = struct.Struct("@qqiiPPPPff")
+_GEMV_TASK = struct.Struct("@iiPPPPiiPP")
+_RTN_TASK = struct.Struct("@qqPiiPPPPPii")
+assert (_MODULE.size, _GEMV_TASK.size, _RTN_TASK.size) == (ct.sizeof(Module), ct.sizeof(GemvTask), ct.sizeof(RtnTask))
+_Tensor = torch.Tensor
+
+
+def _plain(t, dtype, dev: int) -> bool:
+    """A contiguous CUDA tensor of `dtype` on CUDA device `dev`."""
+    return isinstance(t, _Tensor) and t.dtype is dtype and t.is_cuda and t.get_device() == dev and t.is_contiguous()
+
+
+def _pack_modules(modules, decoder: bool):
+    """module_array() and the modules' (rows, cols), or None."""
+    n = len(modules)
+    arr = (Module * n)()
+    size, off, shapes = _MODULE.size, 0, []
+    for m in modules:
+        W0 = m["W0"]
+        if not isinstance(W0, _Tensor) or W0.dim() != 2:
+            return None
+        shape = W0.shape
+        rows, cols = shape
+        dt = W0.dtype
+        code, dev = _WEIGHT_DTYPES.get(dt), W0.get_device()
+        if code is None or not _plain(W0, dt, dev):
+            return None
+        w = act = fisher = wcode = 0
+        if not decoder:
+            W = m.get("W")
+            if W is not None:
+                if not isinstance(W, _Tensor):
+                    return None
+                wdt = W.dtype
+                wcode = _WEIGHT_DTYPES.get(wdt)
+                if wcode is None or not _plain(W, wdt, dev) or W.shape != shape:
+                    return None
+                w = W.data_ptr()
+            a = m.get("act")
+            if a is not None:
+                if not _plain(a, torch.float32, dev) or a.numel() < cols:
+                    return None
+                act = a.data_ptr()
+            f = m.get("fisher")
+            if f is not None:
+                if not _plain(f, torch.float32, dev) or f.shape != shape:
+                    return None
+                fisher = f.data_ptr()
+        _MODULE.pack_into(arr, off, rows, cols, wcode, code, w, W0.data_ptr(), act, fisher,
+                          float(m.get("w_act", 1.0)), float(m.get("w_fisher", 0.0)))
+        off += size
+        shapes.append((rows, cols))
+    return arr, shapes
+
+
+def _modules(modules, decoder: bool = False):
+    """module_array() of the modules and their (rows, cols)."""
+    fast = _pack_modules(modules, decoder)
+    if fast is not None:
+        return fast
+    return module_array(modules, decoder), [_shape(m, i) for i, m in enumerate(modules)]
+
+
+def _pack_shapes(shapes):
+    """shape_modules()."""
+    arr = (Module * len(shapes))()
+    size, off = _MODULE.size, 0
+    for r, c in shapes:
+        _MODULE.pack_into(arr, off, r, c, 0, DTYPE_BF16, 0, 0, 0, 0, 0.0, 0.0)
+        off += size
+    return arr
+
+
+def _pack_gemv(shapes, tasks):
+    """(awsrc_gemv_task[], y's, M) of a batch of products, or None."""
+    arr = (GemvTask * len(tasks))()
+    size, off, ys, M, dev = _GEMV_TASK.size, 0, [], None, None
+    f32, u8 = torch.float32, torch.uint8
+    for t in tasks:
+        if len(t) not in (3, 4):
+            return None
+        m, bb, x = t[0], t[1], t[2]
+        if not isinstance(m, int) or not 0 <= m < len(shapes):
+            return None
+        rows, cols = shapes[m]
+        if not isinstance(x, _Tensor) or x.dim() != 2:
+            return None
+        n, xc = x.shape
+        if dev is None:
+            M, dev = n, x.get_device()
+        if xc != cols or n != M or not _plain(x, f32, dev):
+            return None
+        y = t[3] if len(t) == 4 else None
+        if y is None:
+            y = torch.empty(M, rows, dtype=f32, device=x.device)
+        elif not _plain(y, f32, dev) or tuple(y.shape) != (M, rows):
+            return None
+        G = rows * cols // 128
+        codes = bb["codes"]
+        if not _plain(codes, u8, dev) or codes.numel() < rows * cols // 2:
+            return None
+        if "sdq_codes" in bb:
+            sc, k = bb["sdq_codes"], bb["sdq_consts"]
+            if (not _plain(sc, torch.int8, dev) or sc.numel() < G or not _plain(k, f32, dev) or
+                    k.numel() < 2 * ((G + 255) // 256)):
+                return None
+            pw = (codes.data_ptr(), 0, sc.data_ptr(), k.data_ptr(), 1, 0)
+        else:
+            sc = bb["scales"]
+            if not _plain(sc, torch.int16, dev) or sc.numel() < G:
+                return None
+            pw = (codes.data_ptr(), sc.data_ptr(), 0, 0, 0, 0)
+        _GEMV_TASK.pack_into(arr, off, m, 0, *pw, x.data_ptr(), y.data_ptr())
+        off += size
+        ys.append(y)
+    return arr, ys, M, dev
+
+
+def _pack_rtn(Ws, sdq: bool, outs):
+    """awsrc_rtn_task[] of modules whose outputs the caller holds, or None."""
+    arr = (RtnTask * len(Ws))()
+    size, off = _RTN_TASK.size, 0
+    for W, o in zip(Ws, outs):
+        if not isinstance(W, _Tensor) or W.dim() != 2:
+            return None
+        shape, wdt, dev = W.shape, W.dtype, W.get_device()
+        rows, cols = shape
+        G = rows * cols // 128
+        codes, scales, W0 = o["codes"], o["scales"], o["W0"]
+        if not isinstance(W0, _Tensor):
+            return None
+        wc, w0c = _WEIGHT_DTYPES.get(wdt), _WEIGHT_DTYPES.get(W0.dtype)
+        if (wc is None or w0c is None or not _plain(W, wdt, dev) or not _plain(W0, W0.dtype, dev) or
+                W0.shape != shape or not _plain(codes, torch.uint8, dev) or codes.numel() < rows * cols // 2 or
+                not _plain(scales, torch.int16, dev) or scales.numel() < G):
+            return None
+        sc = k = None
+        if sdq:
+            sc, k = o["sdq_codes"], o["sdq_consts"]
+            if (not _plain(sc, torch.int8, dev) or sc.numel() < G or not _plain(k, torch.float32, dev) or
+                    k.numel() < 2 * ((G + 255) // 256)):
+                return None
+        elif o.get("sdq_codes") is not None or o.get("sdq_consts") is not None:
+            return None
+        _RTN_TASK.pack_into(arr, off, rows, cols, W.data_ptr(), wc, int(sdq), codes.data_ptr(), scales.data_ptr(),
+                            sc.data_ptr() if sdq else 0, k.data_ptr() if sdq else 0, W0.data_ptr(), w0c, 0)
+        off += size
+    return arr
+
+
 def _tiles(prm: Params, modules) -> int:
     return sum(r * c // prm.C for r, c in (_shape(m, i) for i, m in enumerate(modules)))
 
@@ -261,16 +420,18 @@ def awsrc_encode_workspace_bytes(prm: Params, modules) -> int:
 def awsrc_encode_tiles(prm: Params, modules, out: Optional[torch.Tensor] = None,
                        workspace: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """Seed search (Sec. 3.2): one best candidate per tile, uint8 [T, 16] on the device."""
-    T = _tiles(prm, modules)
+    fast = _pack_modules(modules, False)
+    T = _tiles(prm, modules) if fast is None else sum(r * c // prm.C for r, c in fast[1])
     dev = modules[0]["W0"].device
     if out is None:
         out = torch.empty((T, 16), dtype=torch.uint8, device=dev)
     _require(out, "out", dtype=torch.uint8, numel=16 * T, device=dev)
-    mods = module_array(modules)
-    need = awsrc_encode_workspace_bytes(prm, modules)
-    if workspace is None or workspace.numel() < need:
-        workspace = torch.empty(need, dtype=torch.uint8, device=dev)
-    _check(lib.awsrc_encode_tiles(ct.byref(prm), len(modules), mods, _dev_ptr(out), _dev_ptr(workspace),
+    mods = module_array(modules) if fast is None else fast[0]
+    n, p = ct.c_size_t(), ct.byref(prm)
+    _check(lib.awsrc_encode_workspace_bytes(p, len(modules), mods, ct.byref(n)), "encode_workspace_bytes")
+    if workspace is None or workspace.numel() < n.value:
+        workspace = torch.empty(n.value, dtype=torch.uint8, device=dev)
+    _check(lib.awsrc_encode_tiles(p, len(modules), mods, _dev_ptr(out), _dev_ptr(workspace),
                                   workspace.numel(), _stream(stream)), "encode_tiles")
     out._awsrc_workspace = workspace  # keep alive for awsrc_workspace_status
     return out
@@ -325,6 +486,10 @@ def awsrc_rtn_quantize_batch(Ws: Sequence[torch.Tensor], sdq: bool = False, w0_d
     dtypes); returns one output dict per module, as the single call does."""
     if outs is not None and len(outs) != len(Ws):
         raise ValueError(f"{len(outs)} output sets for {len(Ws)} modules")
+    fast = _pack_rtn(Ws, sdq, outs) if outs is not None else None
+    if fast is not None:
+        _check(lib.awsrc_rtn_quantize_batch(len(Ws), fast, _stream(stream)), "rtn_quantize_batch")
+        return list(outs)
     res = [_rtn_buffers(W, sdq, w0_dtype, None if outs is None else outs[i]) for i, W in enumerate(Ws)]
     arr = (RtnTask * len(Ws))()
     for i, (W, o) in enumerate(zip(Ws, res)):
@@ -403,6 +568,14 @@ def awsrc_packed_gemv(prm: Params, shapes, m: int, backbone: Dict[str, torch.Ten
                       stream=None) -> torch.Tensor:
     """y = (W0 + r_hat) x for module m (x: M x cols float32); backbone holds
     awsrc_rtn_quantize's codes and scales (or SDQ codes and constants)."""
+    fast = _pack_gemv(shapes, ((m, backbone, x, y),))
+    if fast is not None and (sidecar is None or _plain(sidecar, torch.uint8, fast[3])):
+        arr = fast[0]
+        _check(lib.awsrc_packed_gemv(ct.byref(prm), len(shapes), _pack_shapes(shapes), m, ct.byref(arr[0].pw),
+                                     None if sidecar is None else sidecar.data_ptr(),
+                                     0 if sidecar is None else sidecar.numel(), fast[2], arr[0].x, arr[0].y,
+                                     _stream(stream)), "packed_gemv")
+        return fast[1][0]
     mods = shape_modules(shapes)
     _require(x, "x", dtype=torch.float32)
     if sidecar is not None:
@@ -418,6 +591,13 @@ def awsrc_packed_gemv_batch(prm: Params, shapes, tasks, sidecar: Optional[torch.
                             stream=None) -> List[torch.Tensor]:
     """Several products in one launch: tasks is a list of (m, backbone, x) or
     (m, backbone, x, y) with the same number M of vectors; returns the y's."""
+    fast = _pack_gemv(shapes, tasks) if tasks else None
+    if fast is not None and (sidecar is None or _plain(sidecar, torch.uint8, fast[3])):
+        _check(lib.awsrc_packed_gemv_batch(ct.byref(prm), len(shapes), _pack_shapes(shapes), len(tasks), fast[0],
+                                           None if sidecar is None else sidecar.data_ptr(),
+                                           0 if sidecar is None else sidecar.numel(), fast[2], _stream(stream)),
+               "packed_gemv_batch")
+        return fast[1]
     mods = shape_modules(shapes)
     if sidecar is not None and tasks:
         _require(tasks[0][2], "x", dtype=torch.float32)
@@ -463,16 +643,19 @@ def awsrc_select_records(prm: Params, modules, cands: torch.Tensor, rates: Seque
     """Sec. 3.3 allocation + Eq. 5 serialisation. Returns (stream bytes [capacity] uint8,
     counts int64 (U: per module, PF: per rate), bytes int64 (per rate)), all on the device.
     Only the first bytes[r] bytes of the stream are written."""
-    _require(cands, "cands", dtype=torch.uint8, numel=16 * _tiles(prm, modules))
+    fast = _pack_modules(modules, True)
+    T = _tiles(prm, modules) if fast is None else sum(r * c // prm.C for r, c in fast[1])
+    _require(cands, "cands", dtype=torch.uint8, numel=16 * T)
     dev = cands.device
     # caller buffers: the stream is bytes, counts and bytes are written as int64
     for name, t, dt in (("out", out, torch.uint8), ("counts", counts, torch.int64), ("nbytes", nbytes, torch.int64)):
         if t is not None:
             _require(t, name, dtype=dt, device=dev)
-    mods = module_array(modules, decoder=True)
+    mods = module_array(modules, decoder=True) if fast is None else fast[0]
     r = (ct.c_double * len(rates))(*rates)
-    cap = awsrc_stream_capacity(prm, modules, rates)
     n = ct.c_size_t()
+    _check(lib.awsrc_stream_capacity(ct.byref(prm), len(modules), mods, r, len(rates), ct.byref(n)), "stream_capacity")
+    cap = n.value
     _check(lib.awsrc_select_workspace_bytes(ct.byref(prm), len(modules), mods, ct.byref(n)), "select_workspace_bytes")
     if workspace is None or workspace.numel() < n.value:
         workspace = torch.empty(n.value, dtype=torch.uint8, device=dev)
@@ -488,6 +671,19 @@ def awsrc_select_records(prm: Params, modules, cands: torch.Tensor, rates: Seque
                                     _dev_ptr(workspace), workspace.numel(), _stream(stream)), "select_records")
     out._awsrc_workspace = workspace
     return out, counts, nbytes
+
+
+def _out_ptrs(modules, outs, dtype):
+    """The outputs' pointers when they pass _check_outs() as they are, else None."""
+    if len(outs) != len(modules):
+        return None
+    ptrs = []
+    for m, o in zip(modules, outs):
+        W0 = m["W0"]
+        if not isinstance(W0, _Tensor) or not _plain(o, dtype, W0.get_device()) or o.shape != W0.shape:
+            return None
+        ptrs.append(o.data_ptr())
+    return (ct.c_void_p * len(ptrs))(*ptrs)
 
 
 def _check_outs(modules, outs, dtype):
@@ -512,9 +708,12 @@ def awsrc_decode_apply(prm: Params, modules, stream_bytes: torch.Tensor, K: int,
     code = DTYPE_F32 if out_dtype == torch.float32 else DTYPE_BF16
     if outs is None:
         outs = [torch.empty_like(m["W0"], dtype=out_dtype) for m in modules]
-    _check_outs(modules, outs, out_dtype)
-    mods = module_array(modules, decoder=True)
-    ptrs = (ct.c_void_p * len(outs))(*[_dev_ptr(o) for o in outs])
+    ptrs = _out_ptrs(modules, outs, out_dtype)
+    if ptrs is None:
+        _check_outs(modules, outs, out_dtype)
+    mods = _modules(modules, decoder=True)[0]
+    if ptrs is None:
+        ptrs = (ct.c_void_p * len(outs))(*[_dev_ptr(o) for o in outs])
     n = ct.c_size_t()
     _check(lib.awsrc_decode_workspace_bytes(ct.byref(prm), len(modules), mods, mode, ct.byref(n)), "decode_workspace_bytes")
     if workspace is None or workspace.numel() < n.value:
