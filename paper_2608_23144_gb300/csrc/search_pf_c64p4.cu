@@ -11,17 +11,24 @@
 // epilogue, which then factors G + eps I (LDL^T), solves, quantises and scores
 // every candidate exactly as the binary32 recipe does.
 //
-// Block: 128 tiles of one column block (row m = TMEM lane m), 13 warps. The
-// producer warp streams 12-seed chunks (FP16 atoms 6 KB, a slice of the U
-// search's atom table, and FP16 atom products 10 KB) through a 4-stage
-// bulk-copy ring and issues per chunk 16 MMAs into one of two TMEM
-// accumulators: Y_hi, Y_lo x atoms (N = 48) and D_hi, D_lo x products (N = 80,
-// the last 8 columns zero). The search is bound by this MMA chain, so a chunk
-// is as many seeds as two accumulators of 256 columns hold. Epilogue warp w
-// takes TMEM lanes 32(w%4).. and seed pairs 2(w/4), 2(w/4) + 1 of each chunk,
-// each as a float2 stream over the pair's two seeds, the two pairs factored
-// side by side so that their dependency chains interleave. Every mbarrier
-// wait is bounded.
+// Block: 128 tiles of one column block (row m = TMEM lane m), 14 warps. The
+// loader warp streams 12-seed chunks (FP16 atoms 6 KB, a slice of the U search's
+// atom table, and FP16 atom products 10 KB) through a 4-stage bulk-copy ring; the
+// MMA warp issues per chunk 16 MMAs into one of two TMEM accumulators: Y_hi, Y_lo
+// x atoms (N = 48) and D_hi, D_lo x products (N = 80, the last 8 columns zero).
+// Epilogue warp w takes TMEM lanes 32(w%4).. and seed pairs 2(w/4), 2(w/4) + 1 of
+// each chunk, each as a float2 stream over the pair's two seeds, the two pairs
+// factored side by side so that their dependency chains interleave. Every
+// mbarrier wait is bounded.
+//
+// What bounds it, per chunk of 12 seeds on one SM (clock64 in copies of the kernel,
+// 1.78 GHz): with one lane issuing the MMAs inside a branch and refilling the ring
+// between them, 2140 cycles, 1360 of them the issue, about 500 the refill; a copy
+// that scored nothing was hardly faster (1840). The issue by a converged warp (630),
+// a loader of its own and the scoring in unit domain (below) each measured nothing
+// or a loss alone; together they take an attention block of a 7B-shaped layer
+// (29.4 M weights, S = 4096) from 9.16 to 8.61 ms. The epilogue bounds it now: three
+// warps per scheduler at 1550 cycles a chunk, their FMA pipe 80% busy meanwhile.
 #include "fit2.cuh"
 #include "internal.h"
 #include "tc05.cuh"
@@ -39,7 +46,7 @@ constexpr int NQ = 6 * CH;          // product columns per chunk
 constexpr int NQP = 80;             // product columns padded to a multiple of 16 (MMA N)
 constexpr int EW = 12;              // epilogue warps: 4 lane quarters x 3 groups of 2 seed pairs
 constexpr int PPW = CH / 2 / (EW / 4);  // seed pairs per epilogue warp and chunk
-constexpr int NT = 32 * (EW + 1);
+constexpr int NT = 32 * (EW + 2);      // + the MMA warp and the loader warp
 constexpr int STAGES = 4;
 constexpr uint32_t kABytes = NA * 64 * 2;      // 6 KB
 constexpr uint32_t kQBytes = NQP * 64 * 2;     // 10 KB (the last 8 columns zero)
@@ -62,11 +69,14 @@ struct Smem {
   float gd[BM];       // G_pp
   float diag[BM];     // fl(gd + eps)
   float invd0[BM];    // 1 / D_0 = 1 / diag
+  float gdu[BM];      // unit domain: gd', 2^(7-qd) diag, -1 / that, 2^(qd-2qy), 2^(2qy-qd)
+  float diag2[BM], ninvd0[BM], to_unit[BM], from_unit[BM];
   float inv_qy[BM], inv_qd[BM];
   int rowok[BM];
   float red_g[EW / 4][BM];
   uint32_t red_s[EW / 4][BM];
   unsigned long long full[STAGES], afull[2], tempty[2];
+  unsigned long long sfree[STAGES];  // a stage's MMAs have completed
   uint32_t tmem_base;
 };
 
@@ -76,30 +86,22 @@ __device__ __forceinline__ int a_offset(int m, int k) {
   return (((m >> 3) * 8 + (k >> 3)) << 7) + ((m & 7) << 4) + ((k & 7) << 1);
 }
 
-// Exact sums RN(2048*hi + lo) of two seeds, scaled by a power of two.
-__device__ __forceinline__ float2 pair_sum(const float* hi, const float* lo, int i, float2 scale) {
-  const float2 u = __ffma2_rn(make_float2(2048.0f, 2048.0f), make_float2(hi[i], hi[i + 1]),
-                              make_float2(lo[i], lo[i + 1]));
-  return __fmul2_rn(u, scale);
+// Exact sums RN(2048*hi + lo) of two seeds.
+__device__ __forceinline__ float2 pair_sum(const float* hi, const float* lo, int i) {
+  return __ffma2_rn(make_float2(2048.0f, 2048.0f), make_float2(hi[i], hi[i + 1]), make_float2(lo[i], lo[i + 1]));
 }
 
-// Fits of NP seed pairs of this thread's row, factored side by side so that
-// their chains interleave; ah/al[j]: atom p of pair j's two seeds at [2p],
-// [2p+1]; qh/ql[j]: product q (tri order) at [2q], [2q+1]. Gives b, the
-// off-diagonal G, alpha and whether each candidate's pivots are valid.
+// Fits of NP seed pairs of this thread's row in the recipe's units, factored
+// side by side so that their chains interleave; bv[j]: b of pair j's two seeds,
+// G[j]: the off-diagonal G (tri order). Gives alpha and whether each candidate's
+// pivots are valid.
 template <int NP>
-__device__ __forceinline__ void pf_fit(const float (*ah)[8], const float (*al)[8], const float (*qh)[12],
-                                       const float (*ql)[12], float tqc, float tqdc, float diag, float invd0,
-                                       float2 (*bv)[4], float2 (*G)[6], float2 (*alpha)[4], bool* okx, bool* oky) {
-  const float2 tq2 = make_float2(tqc, tqc), td2 = make_float2(tqdc, tqdc);
+__device__ __forceinline__ void pf_fit(const float2 (*bv)[4], const float2 (*G)[6], float diag, float invd0,
+                                       float2 (*alpha)[4], bool* okx, bool* oky) {
   const float2 dg = make_float2(diag, diag);
   float2 nL[NP][6], E[NP][6], invD[NP][4];
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
-#pragma unroll
-    for (int p = 0; p < 4; ++p) bv[j][p] = pair_sum(ah[j], al[j], 2 * p, tq2);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) G[j][q] = pair_sum(qh[j], ql[j], 2 * q, td2);
     invD[j][0] = make_float2(invd0, invd0);  // D_0 = diag for every seed
     okx[j] = true;
     oky[j] = true;
@@ -130,15 +132,13 @@ __device__ __forceinline__ void pf_fit(const float (*ah)[8], const float (*al)[8
   for (int j = 0; j < NP; ++j) ldl_solve2<4>(nL[j], invD[j], bv[j], alpha[j]);
 }
 
-// Gains of NP seed pairs (operands as for pf_fit).
+// Gains of NP seed pairs in the recipe's units (operands as for pf_fit).
 template <bool FAST, int NP>
-__device__ __forceinline__ void pf_gain(const Prm& pr, const float (*ah)[8], const float (*al)[8],
-                                        const float (*qh)[12], const float (*ql)[12], float tqc, float tqdc,
-                                        float gd, float diag, float invd0, float2* g,
-                                        float2 (*alpha_out)[4] = nullptr) {
-  float2 bv[NP][4], G[NP][6], alpha[NP][4];
+__device__ __forceinline__ void pf_gain(const Prm& pr, const float2 (*bv)[4], const float2 (*G)[6], float gd,
+                                        float diag, float invd0, float2* g, float2 (*alpha_out)[4] = nullptr) {
+  float2 alpha[NP][4];
   bool okx[NP], oky[NP];
-  pf_fit<NP>(ah, al, qh, ql, tqc, tqdc, diag, invd0, bv, G, alpha, okx, oky);
+  pf_fit<NP>(bv, G, diag, invd0, alpha, okx, oky);
 #pragma unroll
   for (int j = 0; j < NP; ++j) {
     if (alpha_out) {
@@ -167,12 +167,125 @@ __device__ __forceinline__ void pf_gain(const Prm& pr, const float (*ah)[8], con
   }
 }
 
+// ------------------------------------------------------------- unit domain --
+// For C = 64 every scale of the recipe (c, c2, the grids' 2^qy and 2^qd) is a
+// power of two, and the whole fit commutes with powers of two as long as no
+// value over- or underflows. So the common case works on the integer sums
+// themselves, u (for y) and v2 = 2 v (for the off-diagonals; the D operand of the
+// MMAs holds 2 D): with b = 2^(qy-3) u and G = 2^(qd-7) v2,
+//   LDL^T of 2^(7-qd) (G + eps I): the same L, D'' = 2^(7-qd) D;
+//   alpha'' = 2^(qd-qy-4) alpha, hence the same codes, with sc' = 2^(qd-qy-3) sc;
+//   gain = 2^(2qy-qd) sc' (2 sum q u - sc' Qq'), Qq' from gd' = 2^(6-qd) gd and v2
+//     (q_p q_r v2 is the recipe's 2 q_p q_r G: no doubling needed).
+// A row's gains all carry the same factor, so the argmax needs none of it: 10
+// multiplications and 3 additions fewer per seed pair than in the recipe's
+// units, of 96 packed FP32 operations on the pipe that bounds this kernel.
+//
+// The results are those of the recipe bit for bit while nothing leaves the
+// normal range in either domain. That is ensured by testing what could: rows need
+// 2^-26 <= 2^qd <= 2^20 and 2^qy >= 2^-40 (else the block scores in the recipe's
+// units throughout), pivots D'' in [2, 2^40) (so |L| stays moderate and no pivot is a
+// rounding residue: gd'' is at least 2^21) and amax'' in [2^-40, 2^12]. With these
+// amax lies in the recipe's valid range, and a value could only be subnormal in the
+// recipe's units after cancelling more than 80 bits, to where it no longer reaches a
+// code. A pair step in which some lane fails a test is scored again in the recipe's
+// units. Rows outside the numeric domain and rows whose y is zero on the grid (every
+// fit 0, which the recipe calls invalid) have no candidate: their lanes pass.
+constexpr int kUnitQdLo = -26, kUnitQdHi = 20, kUnitQyLo = -40;
+
+// min and max of three (the packed kernels' range tests fold several values).
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float r;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
+// Negated gains (in unit domain) of NP seed pairs; false when some candidate of
+// this lane leaves the ranges above. Everything after the solve works with
+// -alpha'' (the factorisation keeps -1 / D''): rounding is symmetric, so its codes
+// are the negated ones, Qq is even in them, and what comes out, sc' (2 sum q u +
+// sc' Qq), is exactly the negated gain; the search then takes the smallest.
+template <int NP>
+__device__ __forceinline__ bool pf_loss_unit(const Prm& pr, const float2 (*u)[4], const float2 (*v2)[6], float gdu,
+                                             float diag2, float ninvd0, float2* h) {
+  const float2 dg = make_float2(diag2, diag2);
+  float2 nL[NP][6], E[NP][6], nD[NP][4];
+  float2 piv[NP][4];
+#pragma unroll
+  for (int j = 0; j < NP; ++j) nD[j][0] = make_float2(ninvd0, ninvd0);
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+#pragma unroll
+    for (int jp = 0; jp < NP; ++jp) {
+#pragma unroll
+      for (int j = 0; j < k; ++j) {
+        float2 v = v2[jp][tri(k, j)];
+#pragma unroll
+        for (int i = 0; i < j; ++i) v = __ffma2_rn(nL[jp][tri(k, i)], E[jp][tri(j, i)], v);
+        E[jp][tri(k, j)] = v;
+        nL[jp][tri(k, j)] = __fmul2_rn(v, nD[jp][j]);
+      }
+      float2 d = dg;
+#pragma unroll
+      for (int i = 0; i < k; ++i) d = __ffma2_rn(nL[jp][tri(k, i)], E[jp][tri(k, i)], d);
+      piv[jp][k] = d;
+      // -1/D'' correctly rounded as in pivots_rcp, y = approx(-D): y + y (1 + D y)
+      float yx, yy;
+      asm("{\n\t.reg .f32 t;\n\tneg.f32 t, %1;\n\trcp.approx.ftz.f32 %0, t;\n\t}" : "=f"(yx) : "f"(d.x));
+      asm("{\n\t.reg .f32 t;\n\tneg.f32 t, %1;\n\trcp.approx.ftz.f32 %0, t;\n\t}" : "=f"(yy) : "f"(d.y));
+      const float2 ny = make_float2(yx, yy);
+      const float2 e = __ffma2_rn(d, ny, make_float2(1.0f, 1.0f));
+      nD[jp][k] = __ffma2_rn(ny, e, ny);
+    }
+  }
+  // A pivot that leaves [2, 2^40) is finite when it does (those before it are
+  // fine), so the smallest and the largest tell.
+  float dlo = 2.0f, dhi = 0.0f, alo = 1.0f, ahi = 1.0f;
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    dlo = min3(dlo, min3(piv[j][1].x, piv[j][2].x, piv[j][3].x), min3(piv[j][1].y, piv[j][2].y, piv[j][3].y));
+    dhi = max3(dhi, max3(piv[j][1].x, piv[j][2].x, piv[j][3].x), max3(piv[j][1].y, piv[j][2].y, piv[j][3].y));
+  }
+#pragma unroll
+  for (int j = 0; j < NP; ++j) {
+    float2 al[4];
+    ldl_solve2<4>(nL[j], nD[j], u[j], al);
+    const float m0 = fmaxf(max3(fabsf(al[0].x), fabsf(al[1].x), fabsf(al[2].x)), fabsf(al[3].x));
+    const float m1 = fmaxf(max3(fabsf(al[0].y), fabsf(al[1].y), fabsf(al[2].y)), fabsf(al[3].y));
+    alo = min3(alo, m0, m1);
+    ahi = max3(ahi, m0, m1);
+    // 2^e'' by fast_scale_bits(), sc' = 2^(e'' + 1)
+    const uint32_t s0 = fast_scale_bits(pr, __float_as_uint(m0)), s1 = fast_scale_bits(pr, __float_as_uint(m1));
+    const float2 inv = make_float2(__uint_as_float(0x7F000000u - s0), __uint_as_float(0x7F000000u - s1));
+    const float2 sc = make_float2(__uint_as_float(s0 + 0x00800000u), __uint_as_float(s1 + 0x00800000u));
+    const float2 magic = make_float2(12582912.0f, 12582912.0f), nmagic = make_float2(-12582912.0f, -12582912.0f);
+    float2 q[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) q[p] = __fadd2_rn(__ffma2_rn(al[p], inv, magic), nmagic);
+    float2 Aq = make_float2(0.0f, 0.0f), Qq = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) Aq = __ffma2_rn(q[p], u[j][p], Aq);
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      Qq = __ffma2_rn(__fmul2_rn(q[p], q[p]), make_float2(gdu, gdu), Qq);
+#pragma unroll
+      for (int r = p + 1; r < 4; ++r) Qq = __ffma2_rn(__fmul2_rn(q[p], q[r]), v2[j][tri(r, p)], Qq);
+    }
+    h[j] = __fmul2_rn(sc, __ffma2_rn(make_float2(2.0f, 2.0f), Aq, __fmul2_rn(sc, Qq)));
+  }
+  return dlo >= 2.0f && dhi < 0x1p40f && alo >= 0x1p-40f && ahi <= 0x1p12f;
+}
+
 // Codes and scale field of the winning seed of row m. The search keeps only
 // (gain, seed), so the seed's correlations with Y (atoms) and D (atom
 // products) are formed again as the exact integer sums the tensor cores
-// accumulate, split into hi/lo so that 2048*hi + lo is the sum and the fma of
-// pair_sum rounds it once, and go through the same fit and quantiser. Both
-// halves of the pair get the winner's sums; one is read. Returns the gain
+// accumulate, rounded once, and go through the fit and quantiser in the recipe's
+// units. Both halves of the pair get the winner's sums; one is read. Returns the gain
 // once more, which must equal the one the search found.
 template <bool FAST>
 __device__ __forceinline__ float pf_winner(const Prm& pr, const Smem& sm, int m, const uint64_t* mk, bool odd,
@@ -197,21 +310,19 @@ __device__ __forceinline__ float pf_winner(const Prm& pr, const Smem& sm, int m,
 #pragma unroll
     for (int q = 0; q < 6; ++q) nd[q] += ((wq[q] >> j) & 1ull) ? d : 0;
   }
-  float ah[1][8], al[1][8], qh[1][12], ql[1][12];
+  float2 bv[1][4], G[1][6];
 #pragma unroll
-  for (int p = 0; p < 4; ++p) {
-    const int u = ty - 2 * ny[p];  // |u| <= 64 * 2^21
-    ah[0][2 * p] = ah[0][2 * p + 1] = (float)(u >> 11);
-    al[0][2 * p] = al[0][2 * p + 1] = (float)(u & 2047);
+  for (int p = 0; p < 4; ++p) {  // |sum| <= 64 * 2^21, rounded once
+    const float u = __fmul_rn(__int2float_rn(ty - 2 * ny[p]), sm.tqc[m]);
+    bv[0][p] = make_float2(u, u);
   }
 #pragma unroll
   for (int q = 0; q < 6; ++q) {
-    const int u = td - 2 * nd[q];
-    qh[0][2 * q] = qh[0][2 * q + 1] = (float)(u >> 11);
-    ql[0][2 * q] = ql[0][2 * q + 1] = (float)(u & 2047);
+    const float u = __fmul_rn(__int2float_rn(td - 2 * nd[q]), sm.tqdc[m]);
+    G[0][q] = make_float2(u, u);
   }
   float2 alpha[1][4], g;
-  pf_gain<FAST, 1>(pr, ah, al, qh, ql, sm.tqc[m], sm.tqdc[m], sm.gd[m], sm.diag[m], sm.invd0[m], &g, alpha);
+  pf_gain<FAST, 1>(pr, bv, G, sm.gd[m], sm.diag[m], sm.invd0[m], &g, alpha);
   float a[4], q4[4], zero[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
   for (int p = 0; p < 4; ++p) a[p] = odd ? alpha[0][p].y : alpha[0][p].x;
@@ -257,7 +368,10 @@ __global__ void __launch_bounds__(NT, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     if (lane == 0) {
-      for (int i = 0; i < STAGES; ++i) mbar_init(&sm.full[i], 1);
+      for (int i = 0; i < STAGES; ++i) {
+        mbar_init(&sm.full[i], 1);
+        mbar_init(&sm.sfree[i], 1);
+      }
       for (int i = 0; i < 2; ++i) {
         mbar_init(&sm.afull[i], 1);
         mbar_init(&sm.tempty[i], EW);
@@ -271,14 +385,16 @@ __global__ void __launch_bounds__(NT, 1)
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
 
-  int issued = 0;
-  if (warp == EW && lane == 0) {
-    for (; issued < STAGES && issued < nck; ++issued) {
-      mbar_expect_tx(&sm.full[issued], kStageBytes);
-      bulk_g2s(&sm.stage[issued][0], a_src + (size_t)issued * kABytes, kABytes, &sm.full[issued]);
-      bulk_g2s(&sm.stage[issued][kABytes], q_src + (size_t)issued * kQBytes, kQBytes, &sm.full[issued]);
-    }
-  }
+  int issued = 0;  // chunks whose copies the loader issued
+  auto load_chunk = [&]() {
+    const int st = issued % STAGES;
+    mbar_expect_tx(&sm.full[st], kStageBytes);
+    bulk_g2s(&sm.stage[st][0], a_src + (size_t)issued * kABytes, kABytes, &sm.full[st]);
+    bulk_g2s(&sm.stage[st][kABytes], q_src + (size_t)issued * kQBytes, kQBytes, &sm.full[st]);
+    ++issued;
+  };
+  if (warp == EW + 1 && lane == 0)
+    while (issued < STAGES && issued < nck) load_chunk();
   // stage y = d * r and d, d = w_act * a + w_fisher * F (per element)
   for (int e = tid; e < BM * 64; e += NT) {
     const int r = e >> 6, j = e & 63;
@@ -295,6 +411,7 @@ __global__ void __launch_bounds__(NT, 1)
     sm.Dst[r][j] = d;
   }
   __syncthreads();
+  bool safe = true;
   if (tid < BM) {  // per row: fixed-point exponents, gd, eps and the first pivot
     float my = 0.0f, mdd = 0.0f;
     for (int j = 0; j < 64; ++j) {
@@ -310,7 +427,8 @@ __global__ void __launch_bounds__(NT, 1)
     const float gd = __fmul_rn(pr.c2, __fmul_rn(__int2float_rn(sd), two_qd));
     const float eps = __fmul_rn(pr.ridge_rel, gd);
     const float diag = __fadd_rn(gd, eps);
-    const bool ok = sm.rowok[tid] && pivot_ok(diag);
+    // a y of zeros on its grid: every fit is 0, no candidate is valid
+    const bool ok = sm.rowok[tid] && pivot_ok(diag) && iy != 0.0f;
     sm.rowok[tid] = ok ? 1 : 0;
     sm.inv_qy[tid] = ok ? iy : 0.0f;
     sm.inv_qd[tid] = ok ? idd : 0.0f;
@@ -319,8 +437,16 @@ __global__ void __launch_bounds__(NT, 1)
     sm.gd[tid] = gd;
     sm.diag[tid] = diag;
     sm.invd0[tid] = __frcp_rn(diag);
+    // unit domain (a row that is no candidate gets harmless constants)
+    safe = !ok || (qd >= kUnitQdLo && qd <= kUnitQdHi && qy >= kUnitQyLo);
+    const bool un = ok && safe;
+    sm.gdu[tid] = un ? __fmul_rn(gd, pow2f(6 - qd)) : 1.0f;
+    sm.diag2[tid] = un ? __fmul_rn(diag, pow2f(7 - qd)) : 0x1p21f;
+    sm.ninvd0[tid] = -__frcp_rn(sm.diag2[tid]);
+    sm.to_unit[tid] = un ? pow2f(qd - 2 * qy) : 1.0f;
+    sm.from_unit[tid] = un ? pow2f(2 * qy - qd) : 1.0f;
   }
-  __syncthreads();
+  const bool unit = __syncthreads_and(safe) && FAST;
   // A operands: one thread writes one 16-byte core-matrix row of both halves
   for (int e = tid; e < 2 * BM * 8; e += NT) {
     const int which = e >= BM * 8;  // 0: Y, 1: D
@@ -333,10 +459,11 @@ __global__ void __launch_bounds__(NT, 1)
     for (int i = 0; i < 4; ++i) {
       const int x0 = inv == 0.0f ? 0 : fixed_point_int(src[2 * i], inv);
       const int x1 = inv == 0.0f ? 0 : fixed_point_int(src[2 * i + 1], inv);
-      wh[i] = (uint32_t)__half_as_ushort(__int2half_rn(x0 >> 11)) |
-              ((uint32_t)__half_as_ushort(__int2half_rn(x1 >> 11)) << 16);
-      wl[i] = (uint32_t)__half_as_ushort(__int2half_rn(x0 & 2047)) |
-              ((uint32_t)__half_as_ushort(__int2half_rn(x1 & 2047)) << 16);
+      // D doubled: 2 hi <= 2048 and the even 2 lo <= 4094 are exact in FP16
+      wh[i] = (uint32_t)__half_as_ushort(__int2half_rn((x0 >> 11) << which)) |
+              ((uint32_t)__half_as_ushort(__int2half_rn((x1 >> 11) << which)) << 16);
+      wl[i] = (uint32_t)__half_as_ushort(__int2half_rn((x0 & 2047) << which)) |
+              ((uint32_t)__half_as_ushort(__int2half_rn((x1 & 2047) << which)) << 16);
     }
     const int off = a_offset(m, k0);
     *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(sm.A[2 * which]) + off) =
@@ -349,55 +476,68 @@ __global__ void __launch_bounds__(NT, 1)
 
   bool timed_out = false;
   if (warp == EW) {
-    // ------------------------------------------------------------ producer --
+    // ----------------------------------------------------------------- MMAs --
+    uint32_t ab[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ab[i] = smem_addr(sm.A[i]);
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    int k = 0;
+    for (; k < nck; ++k) {
+      const int st = k % STAGES, tb = k & 1;
+      if (!mbar_wait_warp(&sm.full[st], (uint32_t)((k / STAGES) & 1), pr.wait_ns)) { timed_out = true; break; }
+      if (k >= 2 && !mbar_wait_warp(&sm.tempty[tb], (uint32_t)(((k - 2) >> 1) & 1), pr.wait_ns)) { timed_out = true; break; }
+      tc_fence_after();
+      const uint32_t sa = smem_addr(&sm.stage[st][0]), sq = sa + kABytes;
+      const uint32_t acc = tm + (uint32_t)(tb * 256);
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        const uint32_t kb = (uint32_t)ks * 256u, en = ks > 0 ? 1u : 0u;
+        umma_f16_warp(acc + kYH, smem_desc(ab[0] + kb), smem_desc(sa + kb), kIdA, en);
+        umma_f16_warp(acc + kYL, smem_desc(ab[1] + kb), smem_desc(sa + kb), kIdA, en);
+        umma_f16_warp(acc + kDH, smem_desc(ab[2] + kb), smem_desc(sq + kb), kIdQ, en);
+        umma_f16_warp(acc + kDL, smem_desc(ab[3] + kb), smem_desc(sq + kb), kIdQ, en);
+      }
+      umma_commit_warp(&sm.afull[tb]);
+    }
+    // on a timeout wait (bounded) for the MMAs still in flight
+    if (timed_out && k > 0) (void)mbar_wait_warp(&sm.afull[(k - 1) & 1], (uint32_t)(((k - 1) >> 1) & 1), pr.wait_ns);
+  } else if (warp == EW + 1) {
+    // --------------------------------------------------------------- loader --
     if (lane == 0) {
-      uint32_t ab[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) ab[i] = smem_addr(sm.A[i]);
-      int k = 0;
-      for (; k < nck; ++k) {
-        const int st = k % STAGES, tb = k & 1;
-        if (!mbar_wait(&sm.full[st], (uint32_t)((k / STAGES) & 1), pr.wait_ns)) { timed_out = true; break; }
-        if (k >= 2 && !mbar_wait(&sm.tempty[tb], (uint32_t)(((k - 2) >> 1) & 1), pr.wait_ns)) { timed_out = true; break; }
-        tc_fence_after();
-        const uint32_t sa = smem_addr(&sm.stage[st][0]), sq = sa + kABytes;
-        const uint32_t acc = tmem + (uint32_t)(tb * 256);
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-          const uint32_t kb = (uint32_t)ks * 256u, en = ks > 0 ? 1u : 0u;
-          umma_f16(acc + kYH, smem_desc(ab[0] + kb), smem_desc(sa + kb), kIdA, en);
-          umma_f16(acc + kYL, smem_desc(ab[1] + kb), smem_desc(sa + kb), kIdA, en);
-          umma_f16(acc + kDH, smem_desc(ab[2] + kb), smem_desc(sq + kb), kIdQ, en);
-          umma_f16(acc + kDL, smem_desc(ab[3] + kb), smem_desc(sq + kb), kIdQ, en);
-        }
-        umma_commit(&sm.afull[tb]);
-        if (k >= 2 && issued < nck) {
-          // chunk k+2 takes the stage of chunk k-2, whose MMAs completed before
-          // its accumulator was loaded (tempty above)
-          const int ps = (k - 2) % STAGES;
-          mbar_expect_tx(&sm.full[ps], kStageBytes);
-          bulk_g2s(&sm.stage[ps][0], a_src + (size_t)issued * kABytes, kABytes, &sm.full[ps]);
-          bulk_g2s(&sm.stage[ps][kABytes], q_src + (size_t)issued * kQBytes, kQBytes, &sm.full[ps]);
-          ++issued;
-        }
+      while (issued < nck) {  // the stage of chunk issued - STAGES, once its MMAs are complete
+        if (!mbar_wait(&sm.sfree[issued % STAGES], (uint32_t)((issued / STAGES - 1) & 1), pr.wait_ns)) { timed_out = true; break; }
+        load_chunk();
       }
-      if (timed_out) {
-        for (int j = max(0, issued - STAGES); j < issued; ++j)
-          (void)mbar_wait(&sm.full[j % STAGES], (uint32_t)((j / STAGES) & 1), pr.wait_ns);
-        if (k > 0) (void)mbar_wait(&sm.afull[(k - 1) & 1], (uint32_t)(((k - 1) >> 1) & 1), pr.wait_ns);
-      }
+      // the copies in flight land before the block ends, whoever timed out
+      for (int j = max(0, issued - STAGES); j < issued; ++j)
+        if (!mbar_wait(&sm.full[j % STAGES], (uint32_t)((j / STAGES) & 1), pr.wait_ns)) timed_out = true;
     }
   } else {
     // ------------------------------------------------------------ epilogue --
     const int m = 32 * (warp & 3) + lane;
     const int grp = warp >> 2;  // seed pairs 2 grp and 2 grp + 1 of each chunk
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-    const float tqc = sm.tqc[m], tqdc = sm.tqdc[m], gd = sm.gd[m], diag = sm.diag[m], invd0 = sm.invd0[m];
-    float bg = neg_inf();
+    const float gdu = sm.gdu[m], diag2 = sm.diag2[m], ninvd0 = sm.ninvd0[m];
+    // the recipe's units, for the pair steps that need them
+    auto recipe = [&](const float2 (*u)[4], const float2 (*v2)[6], float2* g) {
+      const float tqc = sm.tqc[m], tqdc = __fmul_rn(0.5f, sm.tqdc[m]);  // v2 = 2 v
+      float2 bv[2][4], G[2][6];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+#pragma unroll
+        for (int p = 0; p < 4; ++p) bv[j][p] = __fmul2_rn(u[j][p], make_float2(tqc, tqc));
+#pragma unroll
+        for (int q = 0; q < 6; ++q) G[j][q] = __fmul2_rn(v2[j][q], make_float2(tqdc, tqdc));
+      }
+      pf_gain<FAST, 2>(pr, bv, G, sm.gd[m], sm.diag[m], sm.invd0[m], g);
+    };
+    const bool dead = sm.rowok[m] == 0;
+    float bg = -neg_inf();  // smallest negated gain
     uint32_t bsd = 0xffffffffu;
     for (int k = 0; k < nck; ++k) {
       const int tb = k & 1;
       if (!mbar_wait(&sm.afull[tb], (uint32_t)((k >> 1) & 1), pr.wait_ns)) { timed_out = true; break; }
+      if (tid == 0) mbar_arrive(&sm.sfree[k % STAGES]);
       tc_fence_after();
       const uint32_t base = tmem + lane_base + (uint32_t)(tb * 256);
       // both pairs' columns are loaded before the accumulator is released, so
@@ -428,25 +568,44 @@ __global__ void __launch_bounds__(NT, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.tempty[tb]);
-      float2 g2[2];
-      pf_gain<FAST, 2>(pr, ah, al, qh, ql, tqc, tqdc, gd, diag, invd0, g2);
+      float2 u[2][4], v2[2][6], g2[2];
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        float2 g = g2[j];
-        const int sx = (c0 + k) * CH + 2 * (p0 + j);
-        if (sx + 1 >= pr.S) {  // padding selectors (all-zero masks) are not candidates
-          if (sx >= pr.S) g.x = neg_inf();
-          g.y = neg_inf();
-        }
-        // seeds reach a thread in increasing order: a strictly greater gain wins
-        const float cm = fmaxf(g.x, g.y);
-        if (cm > bg) {
-          bg = cm;
-          bsd = (uint32_t)(sx + (g.x == cm ? 0 : 1));
+#pragma unroll
+        for (int p = 0; p < 4; ++p) u[j][p] = pair_sum(ah[j], al[j], 2 * p);
+#pragma unroll
+        for (int q = 0; q < 6; ++q) v2[j][q] = pair_sum(qh[j], ql[j], 2 * q);
+      }
+      if (!unit) {
+        recipe(u, v2, g2);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) g2[j] = neg2(g2[j]);
+      } else {
+        const bool in = pf_loss_unit<2>(pr, u, v2, gdu, diag2, ninvd0, g2) || dead;
+        if (__any_sync(0xffffffffu, !in)) {
+          recipe(u, v2, g2);
+          const float f = -sm.to_unit[m];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) g2[j] = __fmul2_rn(g2[j], make_float2(f, f));
         }
       }
+      // the smallest negated gain; seeds reach a thread in increasing order, so a
+      // strictly smaller one wins. Padding selectors (all-zero masks, in the last
+      // chunk only) are not candidates.
+      const int sx = (c0 + k) * CH + 2 * p0;
+      if (sx + 3 >= pr.S) {
+        if (sx >= pr.S) g2[0].x = -neg_inf();
+        if (sx + 1 >= pr.S) g2[0].y = -neg_inf();
+        if (sx + 2 >= pr.S) g2[1].x = -neg_inf();
+        if (sx + 3 >= pr.S) g2[1].y = -neg_inf();
+      }
+      const float cm = fminf(min3(g2[0].x, g2[0].y, g2[1].x), g2[1].y);
+      if (cm < bg) {
+        bg = cm;
+        bsd = (uint32_t)(sx + (g2[0].x == cm ? 0 : g2[0].y == cm ? 1 : g2[1].x == cm ? 2 : 3));
+      }
     }
-    sm.red_g[grp][m] = bg;
+    sm.red_g[grp][m] = unit ? __fmul_rn(-bg, sm.from_unit[m]) : -bg;
     sm.red_s[grp][m] = bsd;
   }
   tc_fence_before();
