@@ -8,10 +8,10 @@
 //            array and the tile's map entry (k + 1, seed, scale field) is
 //            raised to it with atomicMax, so a tile named twice is flagged and
 //            takes its later record.
-//   fused    one streaming pass: 16-byte vectors, four in flight per thread
+//   fused    one streaming pass: 16-byte vectors, four in flight per lane
 //            with their tiles' map entries; vectors of unrecorded tiles are
 //            converted and stored at once, those of recorded tiles are queued
-//            in shared memory and patched densely by the whole block:
+//            in shared memory and patched densely by their warp:
 //            W_hat_j = fl(W0_j + fl(fl(k_j * C^-1/2) * scale)) with
 //            k_j = sum_p sign * code_p exact in integers.
 //  in-place mode, and dense mode with tiles shorter than one vector (after a
@@ -440,19 +440,25 @@ __global__ void __launch_bounds__(256) claim_kernel(Prm pr, const __grid_constan
   }
 }
 
-// Dense pass with the patches fused in. A block walks chunks of 1024 vectors (16 bytes each,
-// four per thread, coalesced): vectors of tiles without a record are converted
-// and stored at once; those of recorded tiles (about 16% at 0.162 bits/weight)
-// go, with their W0 data and map entry, to a queue in shared memory that all
-// threads then patch densely. C >= G.
+// Dense pass with the patches fused in. A warp walks chunks of 128 consecutive
+// 16-byte vectors (four per lane, coalesced): vectors of tiles without a record are
+// converted and stored at once; those of recorded tiles (about 16% at 0.162
+// bits/weight) go, with their W0 data and map entry, to the warp's queue in shared
+// memory, which its lanes then patch densely. C >= G. A recorded tile fills
+// neighbouring lanes, so a warp's queue packs its lanes as well as a queue of the
+// whole block did (62 and 64% of them busy at 0.162 bits/weight), and without the
+// block's three barriers per chunk the warps' loads and patches overlap freely:
+// one 3B-shaped layer at 0.162 bits/weight 71.3 -> 68.0 us a decode call, one 7B
+// layer at 0.25 204 -> 191 us, F32 weights 33 -> 27 us (9.4 M of them).
 constexpr int kFusedThreads = 256;
 constexpr int kFusedU = 4;
-constexpr int kFusedChunk = kFusedThreads * kFusedU;
+constexpr int kFusedChunk = 32 * kFusedU;           // vectors per warp and turn
+constexpr int kFusedWarps = kFusedThreads / 32;
 
 struct FusedQ {
   uint4 w0;                 // the vector's W0 bits
   unsigned long long e;     // map entry
-  long long g;              // vector index within the module
+  uint32_t g, pad_;         // vector within the chunk
 };
 
 template <typename TI, typename TO, int G, int PT>
@@ -462,33 +468,33 @@ __global__ void __launch_bounds__(kFusedThreads, 4) fused_kernel(Prm pr, const _
                                                                  const uint64_t* __restrict__ masks,
                                                                  const uint4* __restrict__ nib) {
   static_assert(sizeof(Vec<TI, G>) == 16, "16-byte vectors");
-  __shared__ FusedQ q[kFusedChunk];
-  __shared__ int qn;
+  __shared__ FusedQ queue[kFusedWarps][kFusedChunk];
   const DecodeMod& md = a.m[blockIdx.y];
   const int64_t ngroups = md.rows * md.cols / G;
   const int vshift = pr.logC - (G == 8 ? 3 : 2);  // log2 of the vectors per tile
   const Vec<TI, G>* __restrict__ src = static_cast<const Vec<TI, G>*>(md.W0);
   Vec<TO, G>* __restrict__ dst = static_cast<Vec<TO, G>*>(md.out);
   const unsigned long long* __restrict__ mmap = map + md.tile_off;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  FusedQ* q = queue[warp];
   pdl_wait();  // masks, map and codes come from the preparation kernel
-  for (int64_t c0 = (int64_t)blockIdx.x * kFusedChunk; c0 < ngroups; c0 += (int64_t)gridDim.x * kFusedChunk) {
-    if (threadIdx.x == 0) qn = 0;
-    __syncthreads();
+  const int64_t step = (int64_t)gridDim.x * kFusedWarps * kFusedChunk;
+  for (int64_t c0 = ((int64_t)blockIdx.x * kFusedWarps + warp) * kFusedChunk; c0 < ngroups; c0 += step) {
     Vec<TI, G> v[kFusedU];
     unsigned long long r[kFusedU];
 #pragma unroll
     for (int u = 0; u < kFusedU; ++u) {
-      const int64_t g = c0 + u * kFusedThreads + threadIdx.x;
+      const int64_t g = c0 + u * 32 + lane;
       r[u] = 0ull;
       if (g < ngroups) {
         v[u] = ld_stream(src + g);
         r[u] = __ldg(mmap + (g >> vshift));
       }
     }
+    int n = 0;
 #pragma unroll
     for (int u = 0; u < kFusedU; ++u) {
-      const int64_t g = c0 + u * kFusedThreads + threadIdx.x;
+      const int64_t g = c0 + u * 32 + lane;
       const bool in = g < ngroups;
       const bool patch = in && r[u] != 0ull;
       if (in && !patch) {
@@ -497,28 +503,23 @@ __global__ void __launch_bounds__(kFusedThreads, 4) fused_kernel(Prm pr, const _
         for (int e = 0; e < G; e += 2) Io2<TO>::st(o.v + e, Io2<TI>::ld(v[u].v + e));
         st_stream(dst + g, o);
       }
-      const unsigned m = __ballot_sync(0xffffffffu, patch);  // warp-aggregated append
-      if (m) {
-        int base = 0;
-        if (lane == 0) base = atomicAdd(&qn, __popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (patch) {
-          FusedQ& x = q[base + __popc(m & ((1u << lane) - 1u))];
-          memcpy(&x.w0, &v[u], 16);
-          x.e = r[u];
-          x.g = g;
-        }
+      const unsigned m = __ballot_sync(0xffffffffu, patch);
+      if (patch) {
+        FusedQ& x = q[n + __popc(m & ((1u << lane) - 1u))];
+        memcpy(&x.w0, &v[u], 16);
+        x.e = r[u];
+        x.g = (uint32_t)(u * 32 + lane);
       }
+      n += __popc(m);
     }
-    __syncthreads();
-    const int n = qn;
-    for (int i = threadIdx.x; i < n; i += kFusedThreads) {
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) {
       const FusedQ x = q[i];
       Vec<TI, G> w;
       memcpy(&w, &x.w0, 16);
-      const int64_t k = (int64_t)(x.e >> 32) - 1;
+      const int64_t k = (int64_t)(x.e >> 32) - 1, g = c0 + x.g;
       const uint32_t seed = (uint32_t)(x.e >> 16) & 0xFFFFu;
-      const int j0 = (int)(x.g & ((1 << vshift) - 1)) * G;
+      const int j0 = (int)(g & ((1 << vshift) - 1)) * G;
       Vec<TO, G> o;
       const uint4 slot = __ldg(codes + k);
       const float sc = scale_of(pr, (int16_t)(uint16_t)(x.e & 0xFFFFull));
@@ -528,9 +529,9 @@ __global__ void __launch_bounds__(kFusedThreads, 4) fused_kernel(Prm pr, const _
         patch_vec<TI, TO, G, PT>(pr, w, make_uint2(slot.x, slot.y), masks + (size_t)seed * pr.P * pr.W + (j0 >> 6),
                                  j0, sc, o);
       }
-      st_stream(dst + x.g, o);
+      st_stream(dst + g, o);
     }
-    __syncthreads();
+    __syncwarp();  // the queue is read: the next turn fills it again
   }
 }
 
@@ -595,7 +596,7 @@ cudaError_t launch_fused_t(const Prm& pr, const DecArgs& a, const unsigned long 
   int dev = 0, nsm = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  const int64_t want = (maxg + kFusedChunk - 1) / kFusedChunk;
+  const int64_t want = (maxg + kFusedWarps * kFusedChunk - 1) / (kFusedWarps * kFusedChunk);
   const int64_t gx = std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)nsm * 8));
   const dim3 grid((unsigned)gx, (unsigned)a.n_mod);
   cudaError_t e = pr.P == 4 ? launch_pdl(fused_kernel<TI, TO, G, 4>, grid, dim3(kFusedThreads), st, pr, a, map,
