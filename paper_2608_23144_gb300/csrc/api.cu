@@ -411,7 +411,7 @@ awsrc_status awsrc_gen_basis(const awsrc_params* prm, uint64_t* masks, void* str
   awsrc_status s = make_prm(prm, &pr);
   if (s != AWSRC_OK) return s;
   if (!masks) return AWSRC_ERR_INVALID_ARG;
-  const cudaError_t e = launch_gen_basis(pr, masks, pr.S, (cudaStream_t)stream);
+  const cudaError_t e = launch_gen_basis(pr, masks, pr.S, nullptr, (cudaStream_t)stream);
   return e == cudaSuccess ? AWSRC_OK : cuda_fail(e, "gen_basis");
 }
 
@@ -439,9 +439,7 @@ awsrc_status awsrc_encode_tiles(const awsrc_params* prm, int32_t n_mod, const aw
   awsrc_candidate* pcands = lay.nsplit > 1 ? reinterpret_cast<awsrc_candidate*>(ws + lay.pcands) : out;
   float2* pairs = paired ? reinterpret_cast<float2*>(ws + lay.pairs) : nullptr;
   void* mexp = ws + lay.mexp;
-  cudaError_t e = cudaMemsetAsync(status, 0, sizeof(uint32_t), st);
-  if (e != cudaSuccess) return cuda_fail(e, "encode: clear status");
-  e = launch_gen_basis(pr, masks, pr.S_pad, st);
+  cudaError_t e = launch_gen_basis(pr, masks, pr.S_pad, status, st);
   if (e != cudaSuccess) return cuda_fail(e, "encode: gen_basis");
   void* ptab = ws + lay.ptab;
   if ((lay.spec || lay.spec_pf) && (e = launch_bfrag_c64p4(pr, masks, mexp, st)) != cudaSuccess)

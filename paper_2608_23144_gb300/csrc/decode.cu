@@ -34,13 +34,6 @@ namespace awsrc {
 
 namespace {
 
-// Programmatic dependent launch: a kernel launched with
-// cudaLaunchAttributeProgrammaticStreamSerialization may start while the
-// previous kernel of the stream runs; it must call pdl_wait() before touching
-// anything that kernel writes. pdl_trigger() lets the next kernel launch early.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 struct DecRec {   // an unpacked record; codes packed as signed bytes, code p in byte p
   uint16_t seed;
   int16_t scale;
@@ -545,22 +538,6 @@ __global__ void __launch_bounds__(256) zero_map_kernel(uint4* __restrict__ p, in
     p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// Launch with programmatic serialisation after the previous kernel of `st`.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-}
-
 // Dense-mode preparation for the fused pass: blocks [0, nb) generate the masks
 // (8 warps per block, basis_warp), the remaining blocks fill the tile map
 // (map_records).
@@ -599,9 +576,9 @@ cudaError_t launch_fused_t(const Prm& pr, const DecArgs& a, const unsigned long 
   const int64_t want = (maxg + kFusedWarps * kFusedChunk - 1) / (kFusedWarps * kFusedChunk);
   const int64_t gx = std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)nsm * 8));
   const dim3 grid((unsigned)gx, (unsigned)a.n_mod);
-  cudaError_t e = pr.P == 4 ? launch_pdl(fused_kernel<TI, TO, G, 4>, grid, dim3(kFusedThreads), st, pr, a, map,
+  cudaError_t e = pr.P == 4 ? launch_pdl(fused_kernel<TI, TO, G, 4>, grid, dim3(kFusedThreads), 0, st, pr, a, map,
                                          codes, masks, nib)
-                            : launch_pdl(fused_kernel<TI, TO, G, 0>, grid, dim3(kFusedThreads), st, pr, a, map,
+                            : launch_pdl(fused_kernel<TI, TO, G, 0>, grid, dim3(kFusedThreads), 0, st, pr, a, map,
                                          codes, masks, nib);
   note_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
@@ -716,7 +693,7 @@ cudaError_t launch_dense_prep(const Prm& pr, int64_t T, int64_t L, int64_t h, co
   note_launches(1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = launch_pdl(prep_kernel, dim3((unsigned)(nb + nr)), dim3(256), st, pr, a, stream, masks, map, codes, status,
+  e = launch_pdl(prep_kernel, dim3((unsigned)(nb + nr)), dim3(256), 0, st, pr, a, stream, masks, map, codes, status,
                  nib, nb);
   note_launches(1);
   if (e == cudaSuccess) e = cudaGetLastError();

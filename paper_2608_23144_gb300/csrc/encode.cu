@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(128) gram_u_kernel(Prm pr, LaunchDesc ld,
                                                      const uint64_t* __restrict__ masks,
                                                      float* __restrict__ gram,
                                                      float2* __restrict__ pairs) {
+  pdl_trigger();
   // blockIdx.y enumerates the column blocks of all modules of the launch
   int mi = 0;
   int64_t cb = blockIdx.y;
@@ -141,6 +142,7 @@ __global__ void __launch_bounds__(128) gram_u_kernel(Prm pr, LaunchDesc ld,
     Dt[g][nb] = v;
   }
   __syncthreads();
+  pdl_wait();  // the masks
   // threads past S_pad (the last block of a small S_pad) score a dummy seed
   // whose entries are never written; every thread reaches the barrier below
   const int s_raw = blockIdx.x * blockDim.x + threadIdx.x;
@@ -574,9 +576,9 @@ cudaError_t launch_gram_p(const Prm& pr, const LaunchDesc& ld, const uint64_t* m
   int64_t ncb = 0;
   for (int i = 0; i < ld.n; ++i) ncb += ld.m[i].n_cb;
   dim3 grid((pr.S_pad + 127) / 128, (unsigned)ncb);
-  gram_u_kernel<P><<<grid, 128, 0, st>>>(pr, ld, masks, gram, pairs);
+  const cudaError_t e = launch_pdl(gram_u_kernel<P>, grid, dim3(128), 0, st, pr, ld, masks, gram, pairs);
   note_launches(1);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int P, int VAR>

@@ -4,6 +4,7 @@
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
+#include <utility>
 
 #include "common.cuh"
 
@@ -18,13 +19,44 @@ awsrc_status check_launch(const char* where);
 // Sets the text awsrc_last_error_message() returns (printf-style).
 void set_error_message(const char* fmt, ...);
 
+// Programmatic dependent launch: a kernel launched with launch_pdl() may start
+// while the previous kernel of the stream runs, once every block of that one has
+// called pdl_trigger() or ended; each of its threads must call pdl_wait() before
+// touching anything that kernel (or one before it) writes, or writing anything it
+// reads. Every kernel between two ordinary launches waits, so the chain is in order.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// `early` false: an ordinary launch (the waits then return at once).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dep(bool early, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  return launch_dep(true, kern, grid, block, smem, st, std::forward<Args>(args)...);
+}
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Launch counter behind awsrc_kernel_launches(): every launch site adds its kernels.
 void note_launches(int n);
 
 // masks[(s*P + p)*W + w] for s in [0, S_pad); seeds >= S get zero masks.
-cudaError_t launch_gen_basis(const Prm& pr, uint64_t* masks, int S_out, cudaStream_t st);
+// `status` (may be null): the call's fault word, cleared. The encoder's first
+// launch; those after it are programmatic dependents, up to the merge.
+cudaError_t launch_gen_basis(const Prm& pr, uint64_t* masks, int S_out, uint32_t* status, cudaStream_t st);
 
 
 // encode.cu

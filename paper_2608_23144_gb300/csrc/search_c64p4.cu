@@ -586,6 +586,7 @@ __global__ void __launch_bounds__(NT, 1)
   // compiler keeps the shared address space (LDS/STS, not generic accesses)
   Smem& sm = *reinterpret_cast<Smem*>(smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u));
   const int warp = threadIdx.x >> 5;
+  pdl_trigger();
   if (warp == EW) {  // the producer warp owns the TMEM allocation, held for all tile blocks
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_addr(&sm.tmem_base)),
@@ -593,6 +594,7 @@ __global__ void __launch_bounds__(NT, 1)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  pdl_wait();  // the tables
   for (int64_t blk = blockIdx.x; blk < n_blocks; blk += gridDim.x) {
     if (blk + gridDim.x < n_blocks) prefetch_block(ld, blk + gridDim.x, threadIdx.x);
     // a tile block whose waits ran out ends the CTA's work: its copies or MMAs
@@ -614,6 +616,8 @@ __global__ void __launch_bounds__(NT, 1)
 // i >> 10, column group n8 = (i >> 6) & 15, k group (i >> 3) & 7, row i & 7,
 // and column 8*n8 + r carries atom r >> 1 of seed 32c + 2*n8 + (r & 1).
 __global__ void atoms_kernel(const uint64_t* __restrict__ masks, uint4* __restrict__ out, int S_pad) {
+  pdl_trigger();
+  pdl_wait();  // the masks
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t n = (int64_t)S_pad * 32;
   if (i >= n) return;
@@ -638,7 +642,9 @@ __global__ void merge_kernel(const awsrc_candidate* __restrict__ pc, int nsplit,
                              int64_t t1, awsrc_candidate* __restrict__ out) {
   const int64_t t = t0 + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= t1) return;
+  pdl_wait();  // the search
   awsrc_candidate b = pc[t];
+#pragma unroll 8
   for (int z = 1; z < nsplit; ++z) {
     const awsrc_candidate c = pc[(size_t)z * T + t];
     if (better(c.gain, c.seed, b.gain, b.seed)) b = c;
@@ -654,17 +660,19 @@ size_t search_c64p4_table_bytes(int S_pad) { return (size_t)S_pad * 32 * 16; }
 
 cudaError_t launch_bfrag_c64p4(const Prm& pr, const uint64_t* masks, void* out, cudaStream_t st) {
   const int64_t n = (int64_t)pr.S_pad * 32;
-  atoms_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(masks, static_cast<uint4*>(out), pr.S_pad);
+  const cudaError_t e = launch_pdl(atoms_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, masks,
+                                   static_cast<uint4*>(out), pr.S_pad);
   note_launches(1);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_merge_candidates(const awsrc_candidate* pc, int nsplit, int64_t T, int64_t t0, int64_t t1,
                                    awsrc_candidate* out, cudaStream_t st) {
   if (t1 <= t0) return cudaSuccess;
-  merge_kernel<<<(unsigned)((t1 - t0 + 255) / 256), 256, 0, st>>>(pc, nsplit, T, t0, t1, out);
+  const cudaError_t e = launch_pdl(merge_kernel, dim3((unsigned)((t1 - t0 + 255) / 256)), dim3(256), 0, st, pc, nsplit,
+                                   T, t0, t1, out);
   note_launches(1);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t launch_search_c64p4(const Prm& pr, const LaunchDesc& ld, const void* table,
@@ -679,10 +687,13 @@ cudaError_t launch_search_c64p4(const Prm& pr, const LaunchDesc& ld, const void*
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(n_blocks, nsm));
-  kern<<<(unsigned)grid, NT, smem, st>>>(pr, ld, n_blocks, static_cast<const uint4*>(table), pairs, masks, cands,
-                                         status);
+  // early while the call fits one wave, where launches count (a 256 x 512 matrix with
+  // 256 seeds: 41 -> 31 us with the whole chain early); with more tile blocks the CTAs
+  // that start during the table kernels only disturb them (8661 -> 8686 us a 3B layer)
+  e = launch_dep(n_blocks <= nsm, kern, dim3((unsigned)grid), dim3(NT), smem, st, pr, ld, n_blocks, static_cast<const uint4*>(table),
+                 pairs, masks, cands, status);
   note_launches(1);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace awsrc

@@ -438,7 +438,9 @@ __global__ void __launch_bounds__(32 * kMmaWarps, (VAR == AWSRC_VARIANT_PF && KS
     }
     if (mode == kLoadAsync) asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  pdl_trigger();
   if (blockIdx.x < n_items) fetch(blockIdx.x);
+  pdl_wait();  // the masks and factors; the weights are the caller's, complete since the call's first launch
   for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
     const int z = (int)(item % nsplit);
     const int64_t t0 = first + (item / nsplit) * kMmaTiles + 16 * warp + g;
@@ -596,10 +598,13 @@ cudaError_t launch_mma_t(const Prm& pr, const LaunchDesc& ld, const uint64_t* ma
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(n_items, (int64_t)nsm * per_sm));
-  kern<<<(unsigned)grid, 32 * kMmaWarps, smem, st>>>(pr, ld, masks, reinterpret_cast<const float4*>(pairs), cands,
-                                                     n_items, mode, sl, (int)tab);
+  // early only while every block has an SM of its own: a block that starts beside a
+  // table kernel's finds the SM divided for that kernel, and two per SM then came one
+  // after the other (205 -> 351 us on 9.4 M weights with C = 32, S = 64)
+  e = launch_dep(n_items <= nsm, kern, dim3((unsigned)grid), dim3(32 * kMmaWarps), smem, st, pr, ld, masks,
+                 reinterpret_cast<const float4*>(pairs), cands, n_items, mode, sl, (int)tab);
   note_launches(1);
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int P, int VAR>
