@@ -173,6 +173,20 @@ __device__ __forceinline__ void split4(const float* x, float inv, uint32_t* hi, 
   }
 }
 
+// Largest magnitude of three, ignoring NaN, and propagating it.
+__device__ __forceinline__ float max3_abs(float a, float b, float c) {
+  float r;
+  asm("{\n\t.reg .f32 y, z;\n\tabs.f32 y, %2;\n\tabs.f32 z, %3;\n\tmax.f32 %0, %1, y, z;\n\t}"
+      : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+__device__ __forceinline__ float max3_abs_nan(float a, float b, float c) {
+  float r;
+  asm("{\n\t.reg .f32 y, z;\n\tabs.f32 y, %2;\n\tabs.f32 z, %3;\n\tmax.NaN.f32 %0, %1, y, z;\n\t}"
+      : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 __device__ __forceinline__ float quad_max(float v) {
   v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 1));
   return fmaxf(v, __shfl_xor_sync(0xffffffffu, v, 2));
@@ -234,7 +248,7 @@ __device__ __forceinline__ void mma_stage(const Prm& pr, const LaunchDesc& ld, c
   constexpr bool PF = VAR == AWSRC_VARIANT_PF;
   constexpr int V = KS == 1 ? 4 : 8, NV = 4 * KS / V;
   float y[4 * KS], d[PF ? 4 * KS : 1];
-  // |r| and d over the tile, NaN kept: the tile's domain check is three compares
+  // |r| and |d| over the tile, NaN kept: the tile's domain check is three compares
   float my = 0.0f, mr = 0.0f, dmax = 0.0f, dmin = 0.0f;
   row.pair0 = 0u;
   if (in) {
@@ -279,11 +293,11 @@ __device__ __forceinline__ void mma_stage(const Prm& pr, const LaunchDesc& ld, c
         const float2 yv = __fmul2_rn(dv, r);
         y[v * V + i] = yv.x;
         y[v * V + i + 1] = yv.y;
-        my = fmaxf(my, fmaxf(fabsf(yv.x), fabsf(yv.y)));
-        mr = fmax_nan(mr, fmax_nan(fabsf(r.x), fabsf(r.y)));
-        dmax = fmax_nan(dmax, fmax_nan(dv.x, dv.y));
-        dmin = fminf(dmin, fminf(dv.x, dv.y));
+        my = max3_abs(my, yv.x, yv.y);
+        mr = max3_abs_nan(mr, r.x, r.y);
         if constexpr (PF) {
+          dmax = max3_abs_nan(dmax, dv.x, dv.y);
+          dmin = fminf(dmin, fminf(dv.x, dv.y));
           d[v * V + i] = dv.x;
           d[v * V + i + 1] = dv.y;
         }
@@ -296,7 +310,8 @@ __device__ __forceinline__ void mma_stage(const Prm& pr, const LaunchDesc& ld, c
       if constexpr (PF) d[i] = 0.0f;
     }
   }
-  // in_domain() of every input: |r| <= 2^16 and 0 <= d <= 2^32, no NaN
+  // in_domain() of every input: |r| <= 2^16 and 0 <= d <= 2^32, no NaN (U: an
+  // activation out of range makes its column block's factors invalid)
   bool ok = in && mr <= 65536.0f && dmax <= 4294967296.0f && dmin >= 0.0f;
   // a row's four lanes agree on its grid; a row outside the domain keeps
   // whatever its sums give (rows do not mix) and is dropped at the end
