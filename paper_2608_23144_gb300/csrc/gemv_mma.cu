@@ -27,10 +27,12 @@
 // not depend on what shares its launch.
 //
 // One 3B-shaped layer (77 M weights, 0.162 bits/weight of records, SDQ scales, eight
-// vectors, one batched launch): 263 -> 69 us on the device, 308 -> 76 us a call. Its
+// vectors, one batched launch): 263 -> 66 us on the device, 308 -> 76 us a call. Its
 // relative error against 64 bits is 9.6e-8 where the FP32 pipes' sums had 1.4e-7.
 // Bound by issue (46% of slots): 370 instructions per 16 rows and 128 inputs for the
 // backbone (half of them the split of x) and up to 380 for the residual.
+#include <algorithm>
+
 #include "codetab.cuh"
 #include "internal.h"
 
@@ -316,7 +318,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
 
 }  // namespace
 
-// From three vectors on: the layer of the figures above takes 66 us here whatever
+// From three vectors on: the layer of the figures above takes 65 us here whatever
 // M is, against 30, 47, 125 and 263 us for M = 1, 2, 3 and 8 on the FP32 pipes.
 bool gemv_mma(const Prm& pr, const GemvArgs& a, int M) {
   const bool c = pr.C == 16 || pr.C == 32 || pr.C == 64;
@@ -325,14 +327,24 @@ bool gemv_mma(const Prm& pr, const GemvArgs& a, int M) {
 
 cudaError_t launch_gemv_mma(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st) {
   GemvArgs b = a;
+  // slices of about eight groups (4, 8, 12 and 16 groups measured 70, 66, 66 and 78 us
+  // on the layer above): the shape alone decides, so that a product's sums are the
+  // same in every batch
+  auto slices = [](const GemvTask& t) {
+    const int64_t gpr = t.cols >> 7;
+    int s = 1;
+    while (s < kWarps && gpr > 8 * s) s <<= 1;
+    return s;
+  };
+  // the tasks with the longest slices first, so that their blocks do not end the
+  // launch (69 us in the caller's order, the down projection last)
+  std::stable_sort(b.t, b.t + b.n_task, [&](const GemvTask& x, const GemvTask& y) {
+    return (x.cols >> 7) * slices(y) > (y.cols >> 7) * slices(x);
+  });
   int64_t blocks = 0;
   for (int i = 0; i < b.n_task; ++i) {
     GemvTask& t = b.t[i];
-    // slices of about eight groups: the shape alone decides, so that a product's
-    // sums are the same in every batch
-    const int64_t gpr = t.cols >> 7;
-    t.slices = 1;
-    while (t.slices < kWarps && gpr > 8 * t.slices) t.slices <<= 1;
+    t.slices = slices(t);
     const int64_t per = 16 * (kWarps / t.slices);
     t.block0 = (int)blocks;
     blocks += (t.rows + per - 1) / per;
