@@ -29,10 +29,11 @@
 // Measured on the MLP projections of a 3B-shaped layer (67.6 M weights), whole
 // encode call, against the scalar search that served these shapes before
 // (nibble tables in shared memory, one lane per four seeds): P_F (16, 4, 4, 16)
-// 1832 -> 581 us, U (128, 2, 4, 2) 349 -> 128 us. Loading the next tiles without
-// the copies: 752 and 181 us (40% of the stalls were global loads). P_F is bound by
-// issue (60% of slots; half of the instructions stage and split the inputs, the
-// rest score), U by its loads (110 us of search for 279 MB).
+// 1833 -> 552 us, U (128, 2, 4, 2) 347 -> 98 us. Loading the next tiles without the
+// copies: 752 and 181 us (40% of the stalls were global loads); with the element
+// types tested at run time: 577 and 121 us. P_F is bound by issue (60% of slots; half
+// of the instructions stage and split the inputs, the rest score), U by the latency
+// of its loads and the 16 us of table kernels before it.
 #pragma once
 
 #include <algorithm>
@@ -213,6 +214,17 @@ __device__ __forceinline__ MmaPos mma_pos(const LaunchDesc& ld, int64_t t, int m
   return p;
 }
 
+// The same for tile t, `d` tiles past the one at p0 (one more division only where
+// the step leaves the module or passes a row's end twice).
+__device__ __forceinline__ MmaPos mma_pos_after(const LaunchDesc& ld, const MmaPos& p0, int64_t t, uint32_t d) {
+  const ModDesc& md = ld.m[p0.mi];
+  const uint32_t n_cb = (uint32_t)md.n_cb;
+  MmaPos p{p0.mi, p0.lt + d, p0.cb + d};
+  if (p.cb >= n_cb) p.cb -= n_cb;
+  if (p.cb >= n_cb || (p0.mi + 1 < ld.n && t >= ld.m[p0.mi + 1].tile_off)) p = mma_pos(ld, t, p0.mi);
+  return p;
+}
+
 // What the scoring of one tile needs besides its sums.
 struct MmaRow {
   float tqc;                        // 2^qy c
@@ -222,15 +234,15 @@ struct MmaRow {
 };
 
 // Starts the copies of one tile's inputs into this thread's slots.
-template <int VAR, int KS>
-__device__ __forceinline__ void mma_copy(const Prm& pr, const LaunchDesc& ld, const MmaPos& p, int h, int q,
-                                         const MmaSlots& sl, uint32_t slots) {
+template <int VAR, int KS, bool BF>
+__device__ __forceinline__ void mma_copy(const LaunchDesc& ld, const MmaPos& p, int h, int q, const MmaSlots& sl,
+                                         uint32_t slots) {
   constexpr int V = KS == 1 ? 4 : 8, NV = 4 * KS / V;
   const ModDesc& md = ld.m[p.mi];
-  const int wb = md.w_dtype == AWSRC_DTYPE_F32 ? 4 : 2, w0b = md.w0_dtype == AWSRC_DTYPE_F32 ? 4 : 2;
+  const int wb = !BF && md.w_dtype == AWSRC_DTYPE_F32 ? 4 : 2, w0b = !BF && md.w0_dtype == AWSRC_DTYPE_F32 ? 4 : 2;
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    const int64_t e = (int64_t)p.lt * pr.C + mma_input<KS>(v * (V / 4), q);
+    const uint64_t e = (uint64_t)p.lt * (uint32_t)(16 * KS) + (uint32_t)mma_input<KS>(v * (V / 4), q);
     const uint32_t d = slots + (uint32_t)((h * NV + v) * sl.per_vec) * 512u;
     copy_slots(d + (uint32_t)sl.w * 512u, static_cast<const char*>(md.W) + e * wb, V * wb);
     copy_slots(d + (uint32_t)sl.w0 * 512u, static_cast<const char*>(md.W0) + e * w0b, V * w0b);
@@ -240,7 +252,7 @@ __device__ __forceinline__ void mma_copy(const Prm& pr, const LaunchDesc& ld, co
 
 // Takes one tile's inputs (this thread's 4 KS of C), forms y = d r (and d) on
 // the tile's grid and writes the A fragments of row half `h` (rows g or g + 8).
-template <int P, int VAR, int KS>
+template <int P, int VAR, int KS, bool BF>
 __device__ __forceinline__ void mma_stage(const Prm& pr, const LaunchDesc& ld, const MmaPos& p, bool in, int h, int q,
                                           int mode, const MmaSlots& sl, const unsigned char* slots,
                                           uint32_t (*yh)[4], uint32_t (*yl)[4], uint32_t (*dh)[4], uint32_t (*dl)[4],
@@ -253,24 +265,25 @@ __device__ __forceinline__ void mma_stage(const Prm& pr, const LaunchDesc& ld, c
   row.pair0 = 0u;
   if (in) {
     const ModDesc& md = ld.m[p.mi];
-    const bool bw = md.w_dtype == AWSRC_DTYPE_BF16, bw0 = md.w0_dtype == AWSRC_DTYPE_BF16;
+    const bool bw = BF || md.w_dtype == AWSRC_DTYPE_BF16, bw0 = BF || md.w0_dtype == AWSRC_DTYPE_BF16;
+    constexpr uint32_t C = 16 * KS;
     if constexpr (!PF)
       row.pair0 = (uint32_t)(((uint64_t)md.gram_off + (uint64_t)p.cb * (uint32_t)pr.S_pad) >> 1);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const int j = mma_input<KS>(v * (V / 4), q);
-      const int64_t e = (int64_t)p.lt * pr.C + j;
+      const int64_t e = (int64_t)((uint64_t)p.lt * C + (uint32_t)j);
       float w[V], w0[V], a[V], f[PF ? V : 1];
-      if (mode == kLoadScalar) {
+      if (!BF && mode == kLoadScalar) {
 #pragma unroll
         for (int i = 0; i < V; ++i) {
           w[i] = load_elem(md.W, e + i, md.w_dtype);
           w0[i] = load_elem(md.W0, e + i, md.w0_dtype);
-          a[i] = md.act[p.cb * (uint32_t)pr.C + j + i];
+          a[i] = md.act[p.cb * C + j + i];
           if constexpr (PF) f[i] = md.fisher[e + i];
         }
       } else {
-        if (mode == kLoadAsync) {
+        if (BF || mode == kLoadAsync) {
           const unsigned char* s = slots + (h * NV + v) * sl.per_vec * 512;
           slot_elems<V>(s + sl.w * 512, bw, w);
           slot_elems<V>(s + sl.w0 * 512, bw0, w0);
@@ -280,7 +293,7 @@ __device__ __forceinline__ void mma_stage(const Prm& pr, const LaunchDesc& ld, c
           vec_elems<V>(static_cast<const char*>(md.W0) + e * (bw0 ? 2 : 4), bw0, w0);
           if constexpr (PF) vec_elems<V>(md.fisher + e, false, f);
         }
-        vec_elems<V>(md.act + p.cb * (uint32_t)pr.C + j, false, a);
+        vec_elems<V>(md.act + p.cb * C + j, false, a);
       }
 #pragma unroll
       for (int i = 0; i < V; i += 2) {
@@ -422,7 +435,9 @@ __device__ __forceinline__ void mma_build_table(const Prm& pr, const uint64_t* _
   }
 }
 
-template <int P, int VAR, int KS, bool FAST>
+// BF: W and W0 of every module are BF16 and copied ahead (kLoadAsync), known at
+// compile time.
+template <int P, int VAR, int KS, bool FAST, bool BF>
 __global__ void __launch_bounds__(32 * kMmaWarps, (VAR == AWSRC_VARIANT_PF && KS >= 4) ? 1 : 2)
     search_mma_kernel(Prm pr, const __grid_constant__ LaunchDesc ld, const uint64_t* __restrict__ masks,
                       const float4* __restrict__ pairs, awsrc_candidate* __restrict__ cands, int64_t n_items,
@@ -448,10 +463,11 @@ __global__ void __launch_bounds__(32 * kMmaWarps, (VAR == AWSRC_VARIANT_PF && KS
     const int64_t t0 = first + (item / nsplit) * kMmaTiles + 16 * warp + g;
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
-      pos[r] = mma_pos(ld, min(t0 + 8 * r, last - 1), r ? pos[0].mi : 0);
-      if (mode == kLoadAsync && t0 + 8 * r < last) mma_copy<VAR, KS>(pr, ld, pos[r], r, q, sl, slots_u);
+      const int64_t t = min(t0 + 8 * r, last - 1);
+      pos[r] = r && t == t0 + 8 ? mma_pos_after(ld, pos[0], t, 8u) : mma_pos(ld, t, 0);
+      if ((BF || mode == kLoadAsync) && t0 + 8 * r < last) mma_copy<VAR, KS, BF>(ld, pos[r], r, q, sl, slots_u);
     }
-    if (mode == kLoadAsync) asm volatile("cp.async.commit_group;" ::: "memory");
+    if (BF || mode == kLoadAsync) asm volatile("cp.async.commit_group;" ::: "memory");
   };
   pdl_trigger();
   if (blockIdx.x < n_items) fetch(blockIdx.x);
@@ -461,10 +477,10 @@ __global__ void __launch_bounds__(32 * kMmaWarps, (VAR == AWSRC_VARIANT_PF && KS
     const int64_t t0 = first + (item / nsplit) * kMmaTiles + 16 * warp + g;
     uint32_t yh[KS][4], yl[KS][4], dh[PF ? KS : 1][4], dl[PF ? KS : 1][4];
     MmaRow row[2];
-    if (mode == kLoadAsync) asm volatile("cp.async.wait_all;" ::: "memory");
+    if (BF || mode == kLoadAsync) asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll
     for (int r = 0; r < 2; ++r)
-      mma_stage<P, VAR, KS>(pr, ld, pos[r], t0 + 8 * r < last, r, q, mode, sl, slots, yh, yl, dh, dl, row[r]);
+      mma_stage<P, VAR, KS, BF>(pr, ld, pos[r], t0 + 8 * r < last, r, q, mode, sl, slots, yh, yl, dh, dl, row[r]);
     __syncwarp();  // the slots are read: the next item's copies may start
     if (item + gridDim.x < n_items) fetch(item + gridDim.x);
     float bg[2] = {ninf(), ninf()};
@@ -606,7 +622,10 @@ cudaError_t launch_mma_t(const Prm& pr, const LaunchDesc& ld, const uint64_t* ma
   if (mode == kLoadAsync && smem > kMmaSmemMax) mode = kLoadVector;  // wide F32 tiles
   if (mode != kLoadAsync) smem = tab;
   const int per_sm = most == 2 && 2 * (smem + 1024) <= kMmaSmemMax ? 2 : 1;
-  auto kern = search_mma_kernel<P, VAR, KS, FAST>;
+  // (the binary16-scale and clamped-exponent quantisers keep the one general form)
+  auto kern = search_mma_kernel<P, VAR, KS, FAST, false>;
+  if constexpr (FAST)
+    if (mode == kLoadAsync && wb == 2 && w0b == 2) kern = search_mma_kernel<P, VAR, KS, FAST, true>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMmaSmemMax);
   if (e != cudaSuccess) return e;
   int dev = 0, nsm = 0;
