@@ -73,20 +73,10 @@ __device__ __forceinline__ bool split_run(const float4& xa, const float4& xb, BR
     const float2 s = __fadd2_rn(r[i], make_float2(-upper(r[i].x), -upper(r[i].y)));
     b.lo[i] = upper_pair(s.x, s.y);
   }
-  // an infinity or NaN leaves a NaN remainder: keep it in hi alone, so that it
-  // enters the products once, as itself
+  // an infinity or NaN leaves a NaN remainder
   const float2 t = __fadd2_rn(__fadd2_rn(r[0], r[1]), __fadd2_rn(r[2], r[3]));
   const float n = __fadd_rn(t.x, t.y);
-  if (n != n) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      b.hi[i] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(a[i])) |
-                ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(c[i])) << 16);
-      b.mid[i] = b.lo[i] = 0u;
-    }
-    return true;
-  }
-  return false;
+  return n != n;
 }
 
 // Codes i and i + 4 of a code word as a BF16 pair: 128 + u (u = code + 8) in the
@@ -150,6 +140,47 @@ __device__ __forceinline__ void residual_pairs(const TileRec& t, const uint4& nb
     uint32_t d;
     asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(v), "r"(0x43404340u));
     asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r[i]) : "r"(d), "r"(t.sc));
+  }
+}
+
+// A run's products with the vectors named by `odd` (any of a quad's four bits: that
+// quad's vector), on the FP32 pipes as gemv.cu forms them: x, the thread's inputs of
+// vector 0; r0, r1, its A pairs of rows g and g + 8, left out where use0, use1 are
+// false. out: the run's sums of rows g, g + 8 and vectors 2q, 2q + 1, like an MMA's.
+__device__ __forceinline__ void run_fp32(const float* x, int64_t cols, unsigned odd, int q, const uint32_t (&r0)[4],
+                                         const uint32_t (&r1)[4], bool use0, bool use1, float (&out)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) out[i] = 0.0f;
+#pragma unroll 1
+  for (int n = 0; n < 8; ++n) {
+    if (((odd >> (4 * n)) & 15u) == 0u) continue;
+    const float4 xa = __ldg(reinterpret_cast<const float4*>(x + n * cols));
+    const float4 xb = __ldg(reinterpret_cast<const float4*>(x + n * cols + 4));
+    const float v[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+    float p0 = 0.0f, p1 = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      p0 = __fmaf_rn(__uint_as_float(r0[i] << 16), v[i], p0);
+      p0 = __fmaf_rn(upper(__uint_as_float(r0[i])), v[i + 4], p0);
+      p1 = __fmaf_rn(__uint_as_float(r1[i] << 16), v[i], p1);
+      p1 = __fmaf_rn(upper(__uint_as_float(r1[i])), v[i + 4], p1);
+    }
+    if (!use0) p0 = 0.0f;
+    if (!use1) p1 = 0.0f;
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+      p0 = __fadd_rn(p0, __shfl_xor_sync(0xffffffffu, p0, off));
+      p1 = __fadd_rn(p1, __shfl_xor_sync(0xffffffffu, p1, off));
+    }
+    if (q == n >> 1) {
+      if (n & 1) {
+        out[1] = p0;
+        out[3] = p1;
+      } else {
+        out[0] = p0;
+        out[2] = p1;
+      }
+    }
   }
 }
 
@@ -241,43 +272,38 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
         for (int r = 0; r < 2; ++r) nb[r] = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + win);
       }
       BRun b;
-      const bool bad = split_run(xa, xb, b);
+      // Vectors with an infinity or NaN in this run: no MMA may see them, since a row
+      // whose A is zero there (no record, or another tile's lanes) would get 0 * infinity
+      const unsigned odd = __ballot_sync(0xffffffffu, split_run(xa, xb, b));
+      const float* xr = tk.x + 128 * gr + 32 * j + 8 * q;
+      if (odd && ((odd >> (lane & 28)) & 15u) != 0u) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) b.hi[i] = b.mid[i] = b.lo[i] = 0u;
+      }
       uint32_t c0[4], c1[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         c0[i] = code_pair(wc[0][j], i);
         c1[i] = code_pair(wc[1][j], i);
       }
+      if (odd) {
+        float o[4];
+        run_fp32(xr, tk.cols, odd, q, c0, c1, true, true, o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (sc[i >> 1] != 0.0f) acc[i] = __fmaf_rn(o[i], sc[i >> 1], acc[i]);
+      }
       mma_run(h, ml, c0, c1, b);
       if (any) {
         residual_pairs(tr[0], nb[0], c0);
         residual_pairs(tr[1], nb[1], c1);
-        if (!__any_sync(0xffffffffu, bad)) {
-          mma_run(rh, rml, c0, c1, b);
-        } else {
-          // a row without a record here must not meet 0 * infinity: the inputs of
-          // lanes with one go apart and count for recorded rows only
-          float th[4] = {0.0f, 0.0f, 0.0f, 0.0f}, tm[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-          BRun fin;
+        if (odd) {
+          float o[4];
+          run_fp32(xr, tk.cols, odd, q, c0, c1, ec[0][t] != 0ull, ec[1][t] != 0ull, o);
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            fin.hi[i] = bad ? 0u : b.hi[i];
-            fin.mid[i] = bad ? 0u : b.mid[i];
-            fin.lo[i] = bad ? 0u : b.lo[i];
-            b.hi[i] = bad ? b.hi[i] : 0u;
-            b.mid[i] = b.lo[i] = 0u;
-          }
-          mma_run(rh, rml, c0, c1, fin);
-          mma_run(th, tm, c0, c1, b);
-#pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            const unsigned has = __ballot_sync(0xffffffffu, ec[r][t] != 0ull) >> (lane & 28) & 15u;
-            if (has) {
-              racc[2 * r] = __fadd_rn(racc[2 * r], __fadd_rn(th[2 * r], tm[2 * r]));
-              racc[2 * r + 1] = __fadd_rn(racc[2 * r + 1], __fadd_rn(th[2 * r + 1], tm[2 * r + 1]));
-            }
-          }
+          for (int i = 0; i < 4; ++i) racc[i] = __fadd_rn(racc[i], o[i]);
         }
+        mma_run(rh, rml, c0, c1, b);
       }
     }
 #pragma unroll

@@ -1,0 +1,66 @@
+"""The packed product of three to eight vectors on inputs at the ends of binary32's
+range, against the one-vector kernel and the oracle's double-precision definition."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _bound(cols, C, yabs):
+    """The header's bound, without slack: (cols / min(C, 32) + 32) * 2^-24 * sum_j (|W0 x| + |r x|)."""
+    return (cols / min(C, 32) + 32) * 2.0 ** -24 * yabs
+
+
+def _setup(aw, orc, kw, W, recorded, scale, codes, rng):
+    """Backbone of W, and a prepared sidecar that names the tiles of `recorded` (bool per tile)."""
+    shapes = [W.shape]
+    obb = orc.rtn_quantize(W, sdq=False)
+    prm, oprm = aw.params(**kw), orc.params(**kw)
+    T = W.size // prm.C
+    c = np.zeros(T, aw.CANDIDATE_DTYPE)
+    c["gain"][recorded] = 1.0
+    c["seed"] = rng.integers(0, prm.S, T)
+    c["scale"] = scale
+    c["code"][:, :4] = codes(T)
+    stream, counts, _ = orc.select_records(oprm, shapes, c, [40.0])
+    K = int(counts.sum())
+    assert K == recorded.sum()
+    side = aw.awsrc_sidecar_prepare(prm, shapes, torch.from_numpy(np.frombuffer(stream, np.uint8).copy()).cuda(), K)
+    bb = aw.awsrc_rtn_quantize(torch.from_numpy(W).cuda())
+
+    def gemv(x):
+        return aw.awsrc_packed_gemv(prm, shapes, 0, bb, torch.from_numpy(x).cuda(), sidecar=side).cpu().numpy()
+
+    def definition(x):
+        y, yabs, bad = orc.packed_gemv(oprm, obb["q"], obb["s_eff"], 128, stream, K, x, shapes=shapes, m=0)
+        assert bad == 0
+        return y, yabs
+    return gemv, definition
+
+
+@pytest.mark.parametrize("C", [16, 32, 64])
+def test_infinity_beside_recorded_tiles(orc, C):
+    """Every other tile recorded, the infinities and NaN in tiles without a record: the
+    recorded neighbour's row takes the backbone's infinity, or (scale 0) nothing."""
+    import paper_2608_23144_gb300 as aw
+    rng = np.random.default_rng(51)
+    rows, cols, M = 48, 256, 5
+    W = rng.normal(0, 0.02, (rows, cols)).astype(np.float32)
+    W[::3, :128] = 0.0  # groups of scale 0
+    even = np.arange(W.size // C) % 2 == 0
+    gemv, _ = _setup(aw, orc, dict(C=C, P=4, b=4, S=64), W, even, -8, lambda T: rng.integers(-7, 8, (T, 4)), rng)
+    x = rng.normal(0, 1, (M, cols)).astype(np.float32)
+    clean = x.copy()
+    x[1, C + 3] = np.inf
+    x[2, 2 * C - 1] = -np.inf
+    x[3, C] = np.nan
+    y, yc = gemv(x), gemv(clean)
+    one = np.concatenate([gemv(x[v:v + 1]) for v in range(M)])
+    assert np.isfinite(one[1, ::3]).all() and np.isfinite(one[3, ::3]).all() and np.isinf(one[1]).any()
+    for v in (0, 4):
+        assert np.array_equal(y[v], yc[v])
+    assert np.array_equal(np.isnan(y), np.isnan(one))
+    assert np.array_equal(np.isposinf(y), np.isposinf(one)) and np.array_equal(np.isneginf(y), np.isneginf(one))
+    fin = np.isfinite(one)
+    assert np.allclose(y[fin], one[fin], rtol=1e-5, atol=1e-5)
