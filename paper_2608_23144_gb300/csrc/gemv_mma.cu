@@ -12,7 +12,8 @@
 //    mask-and-xor into the mantissa of 128 + u and one packed subtraction;
 //  * B: x as x = hi + mid + lo, three BF16 numbers whose sum is x exactly (8 + 8 + 8
 //    significand bits by truncation), so a product loses nothing that binary32
-//    holds; the chain of the hi parts and that of the mid and lo parts have their own
+//    holds. Where it is not (an input below 2^-110 whose last bits BF16 cannot hold, an
+//    infinity or NaN) the vector's run goes through the FP32 pipes instead. The chain of the hi parts and that of the mid and lo parts have their own
 //    binary32 accumulators, over one group of 128 inputs each. A group's sum is
 //    multiplied by its scale and added with binary32 FMAs, as before.
 //  * The residual: k_j c 2^e is exact in BF16 (|k_j| <= 64), so recorded tiles are a
@@ -61,22 +62,22 @@ struct BRun {
   uint32_t hi[4], mid[4], lo[4];
 };
 
-// Returns whether one of the eight inputs is an infinity or NaN.
+// Returns whether the three parts of each input are the input. They are from 2^-110
+// on; below, an input may have bits under 2^-133, which BF16 has not, and an infinity
+// or NaN leaves a NaN: either way what is left of the third part has low bits.
 __device__ __forceinline__ bool split_run(const float4& xa, const float4& xb, BRun& b) {
   const float a[4] = {xa.x, xa.y, xa.z, xa.w}, c[4] = {xb.x, xb.y, xb.z, xb.w};
-  float2 r[4];
+  uint32_t left = 0u;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     b.hi[i] = upper_pair(a[i], c[i]);
-    r[i] = __fadd2_rn(make_float2(a[i], c[i]), make_float2(-upper(a[i]), -upper(c[i])));
-    b.mid[i] = upper_pair(r[i].x, r[i].y);
-    const float2 s = __fadd2_rn(r[i], make_float2(-upper(r[i].x), -upper(r[i].y)));
+    const float2 r = __fadd2_rn(make_float2(a[i], c[i]), make_float2(-upper(a[i]), -upper(c[i])));
+    b.mid[i] = upper_pair(r.x, r.y);
+    const float2 s = __fadd2_rn(r, make_float2(-upper(r.x), -upper(r.y)));
     b.lo[i] = upper_pair(s.x, s.y);
+    left |= __float_as_uint(s.x) | __float_as_uint(s.y);
   }
-  // an infinity or NaN leaves a NaN remainder
-  const float2 t = __fadd2_rn(__fadd2_rn(r[0], r[1]), __fadd2_rn(r[2], r[3]));
-  const float n = __fadd_rn(t.x, t.y);
-  return n != n;
+  return (left & 0xFFFFu) == 0u;
 }
 
 // Codes i and i + 4 of a code word as a BF16 pair: 128 + u (u = code + 8) in the
@@ -272,9 +273,10 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
         for (int r = 0; r < 2; ++r) nb[r] = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + win);
       }
       BRun b;
-      // Vectors with an infinity or NaN in this run: no MMA may see them, since a row
-      // whose A is zero there (no record, or another tile's lanes) would get 0 * infinity
-      const unsigned odd = __ballot_sync(0xffffffffu, split_run(xa, xb, b));
+      // Vectors that the MMAs cannot take in this run: inputs too small for the split, or
+      // an infinity or NaN (a row whose A is zero there, with no record or in another
+      // tile's lanes, would get 0 * infinity)
+      const unsigned odd = __ballot_sync(0xffffffffu, !split_run(xa, xb, b));
       const float* xr = tk.x + 128 * gr + 32 * j + 8 * q;
       if (odd && ((odd >> (lane & 28)) & 15u) != 0u) {
 #pragma unroll

@@ -64,3 +64,25 @@ def test_infinity_beside_recorded_tiles(orc, C):
     assert np.array_equal(np.isposinf(y), np.isposinf(one)) and np.array_equal(np.isneginf(y), np.isneginf(one))
     fin = np.isfinite(one)
     assert np.allclose(y[fin], one[fin], rtol=1e-5, atol=1e-5)
+
+
+@pytest.mark.parametrize("C,scale", [(64, -8), (64, 90), (32, -8), (16, 90)])
+def test_small_inputs(orc, C, scale):
+    """Inputs from 2^-100 down to the subnormals, where x has bits that BF16 does not:
+    the header's bound relative to the products themselves (which large record scales
+    bring back into the ordinary range). All of one sign, so that lost bits add up.
+    Below the normal range each of the bound's roundings may also lose half of 2^-149."""
+    import paper_2608_23144_gb300 as aw
+    rng = np.random.default_rng(61)
+    rows, cols, M = 40, 384, 8
+    W = np.abs(rng.normal(0, 0.02, (rows, cols))).astype(np.float32) + np.float32(0.01)
+    gemv, definition = _setup(aw, orc, dict(C=C, P=4, b=4, S=64), W, rng.random(W.size // C) < 0.5, scale,
+                              lambda T: rng.integers(1, 8, (T, 4)), rng)
+    x = rng.uniform(1, 2, (M, cols))
+    x *= 2.0 ** np.array([-100, -108, -111, -114, -118, -122, -130, 0])[:, None]
+    x[7] *= 2.0 ** rng.integers(-140, 1, cols)  # every magnitude in one vector
+    x = x.astype(np.float32)
+    y = gemv(x)
+    want, yabs = definition(x)
+    err = np.abs(y - want)
+    assert (err <= _bound(cols, C, yabs) + (cols / min(C, 32) + 32) * 2.0 ** -150).all(), (err / yabs).max(1) * 2 ** 24
