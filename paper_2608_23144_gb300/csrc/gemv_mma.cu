@@ -103,7 +103,8 @@ __device__ __forceinline__ void mma_run(float (&h)[4], float (&ml)[4], const uin
 
 // What a thread needs of a recorded tile of its row: the record's byte tables as
 // k_j + 64, and 2^(e - S) in both halves of a BF16 pair (k_j 2^(e - S) is k_j c 2^e
-// for C = 64 and 16, k_j 2^e / 4 for C = 32; 2^(e - S) may be a subnormal BF16).
+// for C = 64 and 16, k_j 2^e / 8 for C = 32, which is finite where k_j c 2^e is;
+// 2^(e - S) may be a subnormal BF16).
 struct TileRec {
   KTab kt;
   uint32_t sc;
@@ -118,7 +119,7 @@ __device__ __forceinline__ TileRec tile_rec(const GemvArgs& a, unsigned long lon
   // k_tables() gives k + 128 as bytes of 64 .. 192
   const KTab k = k_tables(slot);
   t.kt = {k.t0 - 0x40404040u, k.t1 - 0x40404040u, k.u0 - 0x40404040u, k.u1 - 0x40404040u};
-  constexpr int S = LC == 6 ? 3 : 2;
+  constexpr int S = LC == 4 ? 2 : 3;
   const int f = (int)(int16_t)(uint16_t)(e & 0xFFFFull) - S;
   const uint32_t sb = f >= -126 ? (uint32_t)(f + 127) << 7 : 1u << (f + 133);
   t.sc = sb * 0x00010001u;
@@ -316,8 +317,8 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
       racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
     }
   }
-  // c = 2^-(LC/2) is folded into the residual for C = 64 and 16; C = 32 had 1/4
-  const float cf = LC == 5 ? __fmul_rn(4.0f, pr.c) : 1.0f;
+  // c = 2^-(LC/2) is folded into the residual for C = 64 and 16; C = 32 had 1/8
+  const float cf = LC == 5 ? __fmul_rn(8.0f, pr.c) : 1.0f;
   float v[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) v[i] = __fmaf_rn(racc[i], cf, acc[i]);

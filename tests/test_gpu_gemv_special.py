@@ -86,3 +86,21 @@ def test_small_inputs(orc, C, scale):
     want, yabs = definition(x)
     err = np.abs(y - want)
     assert (err <= _bound(cols, C, yabs) + (cols / min(C, 32) + 32) * 2.0 ** -150).all(), (err / yabs).max(1) * 2 ** 24
+
+
+@pytest.mark.parametrize("C", [16, 32, 64])
+def test_largest_record_scale(orc, C):
+    """The residual's operand k_j c 2^e near binary32's largest number (e = 126, and
+    |k_j c| < 4) is finite, hence so is its product with small inputs."""
+    import paper_2608_23144_gb300 as aw
+    rng = np.random.default_rng(81)
+    rows, cols, M = 40, 256, 3
+    q = {16: 3, 32: 5, 64: 7}[C]  # |k_j| <= 4 q: k_j c up to 3, 3.5, 3.5
+    W = rng.normal(0, 0.02, (rows, cols)).astype(np.float32)
+    gemv, definition = _setup(aw, orc, dict(C=C, P=4, b=4, S=64), W, rng.random(W.size // C) < 0.5, 126,
+                              lambda T: q * rng.choice([-1, 1], (T, 4)), rng)
+    x = (rng.uniform(-1, 1, (M, cols)) * 2.0 ** -40).astype(np.float32)
+    y = gemv(x)
+    want, yabs = definition(x)
+    assert np.isfinite(gemv(x[:1])).all() and np.abs(want).max() > 2.0 ** 80
+    assert (np.abs(y - want) <= _bound(cols, C, yabs)).all()
