@@ -12,10 +12,12 @@
 //    mask-and-xor into the mantissa of 128 + u and one packed subtraction;
 //  * B: x as x = hi + mid + lo, three BF16 numbers whose sum is x exactly (8 + 8 + 8
 //    significand bits by truncation), so a product loses nothing that binary32
-//    holds. Where it is not (an input below 2^-110 whose last bits BF16 cannot hold, an
-//    infinity or NaN) the vector's run goes through the FP32 pipes instead. The chain of the hi parts and that of the mid and lo parts have their own
-//    binary32 accumulators, over one group of 128 inputs each. A group's sum is
-//    multiplied by its scale and added with binary32 FMAs, as before.
+//    holds. Where it is not (an input below 2^-110 whose last bits BF16 cannot hold,
+//    an infinity or NaN) the vector's run goes through the FP32 pipes instead. The
+//    chain of the hi parts and that of the mid and lo parts have their own binary32
+//    accumulators, over one run of 32 inputs each: the sums that gemv.cu's lanes form,
+//    which overflow only where those do. A run's sum is multiplied by its group's scale
+//    and added with binary32 FMAs.
 //  * The residual: k_j c 2^e is exact in BF16 (|k_j| <= 64), so recorded tiles are a
 //    second A operand against the same B (rows without a record: zeros), with its own
 //    accumulators; column runs without any record in the 16 rows are skipped.
@@ -248,7 +250,6 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
       for (int t = 0; t < NT; ++t) ec[r][t] = e[r][t];
     }
     if (gr + 1 < g1) load(gr + 1);
-    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     float rh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     TileRec tr[2];
     bool any = false;
@@ -296,7 +297,11 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
         for (int i = 0; i < 4; ++i)
           if (sc[i >> 1] != 0.0f) acc[i] = __fmaf_rn(o[i], sc[i >> 1], acc[i]);
       }
+      float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
       mma_run(h, ml, c0, c1, b);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)  // an all-zero group (scale 0) adds nothing, whatever x holds
+        if (sc[i >> 1] != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sc[i >> 1], acc[i]);
       if (any) {
         residual_pairs(tr[0], nb[0], c0);
         residual_pairs(tr[1], nb[1], c1);
@@ -310,12 +315,7 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
       }
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      // an all-zero group (scale 0) adds nothing, whatever x holds
-      const float sr = sc[i >> 1];
-      if (sr != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sr, acc[i]);
-      racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
-    }
+    for (int i = 0; i < 4; ++i) racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
   }
   // c = 2^-(LC/2) is folded into the residual for C = 64 and 16; C = 32 had 1/8
   const float cf = LC == 5 ? __fmul_rn(8.0f, pr.c) : 1.0f;

@@ -88,6 +88,23 @@ def test_small_inputs(orc, C, scale):
     assert (err <= _bound(cols, C, yabs) + (cols / min(C, 32) + 32) * 2.0 ** -150).all(), (err / yabs).max(1) * 2 ** 24
 
 
+def test_large_inputs(orc):
+    """Codes of 7 throughout and inputs at which a sum over a group's 128 codes and
+    inputs would overflow, though one over 32 does not and the product, after the
+    group's scale, is far from it."""
+    import paper_2608_23144_gb300 as aw
+    rng = np.random.default_rng(71)
+    rows, cols, M, C = 40, 256, 3, 64
+    W = np.full((rows, cols), 0.02, np.float32)
+    gemv, definition = _setup(aw, orc, dict(C=C, P=4, b=4, S=64), W, rng.random(W.size // C) < 0.5, -10,
+                              lambda T: rng.integers(-7, 8, (T, 4)), rng)
+    x = rng.uniform(0.9e36, 1.2e36, (M, cols)).astype(np.float32)
+    y = gemv(x)
+    want, yabs = definition(x)
+    assert np.isfinite(want).all() and np.isfinite(np.concatenate([gemv(x[v:v + 1]) for v in range(M)])).all()
+    assert (np.abs(y - want) <= _bound(cols, C, yabs)).all()
+
+
 @pytest.mark.parametrize("C", [16, 32, 64])
 def test_largest_record_scale(orc, C):
     """The residual's operand k_j c 2^e near binary32's largest number (e = 126, and
