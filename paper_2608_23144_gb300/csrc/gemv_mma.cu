@@ -13,11 +13,12 @@
 //  * B: x as x = hi + mid + lo, three BF16 numbers whose sum is x exactly (8 + 8 + 8
 //    significand bits by truncation), so a product loses nothing that binary32
 //    holds. Where it is not (an input below 2^-110 whose last bits BF16 cannot hold,
-//    an infinity or NaN) the vector's run goes through the FP32 pipes instead. The
+//    an infinity or NaN), or a group's sum could overflow where gemv.cu's lanes, which
+//    sum 32 inputs, do not, the vector's group goes through the FP32 pipes instead. The
 //    chain of the hi parts and that of the mid and lo parts have their own binary32
-//    accumulators, over one run of 32 inputs each: the sums that gemv.cu's lanes form,
-//    which overflow only where those do. A run's sum is multiplied by its group's scale
-//    and added with binary32 FMAs.
+//    accumulators, over one group of 128 inputs each (sums of 32 added with FMAs had a
+//    relative error of 1.4e-7 where these have 9.9e-8). A group's sum is multiplied by
+//    its scale and added with binary32 FMAs.
 //  * The residual: k_j c 2^e is exact in BF16 (|k_j| <= 64), so recorded tiles are a
 //    second A operand against the same B (rows without a record: zeros), with its own
 //    accumulators; column runs without any record in the 16 rows are skipped.
@@ -58,28 +59,43 @@ __device__ __forceinline__ uint32_t upper_pair(float a, float b) {
 }
 __device__ __forceinline__ float upper(float a) { return __uint_as_float(__float_as_uint(a) & 0xffff0000u); }
 
+// Largest magnitude, of numbers.
+__device__ __forceinline__ float max3_abs(float m, float a, float b) {
+  float r;
+  asm("{\n\t.reg .f32 y, z;\n\tabs.f32 y, %2;\n\tabs.f32 z, %3;\n\tmax.f32 %0, %1, y, z;\n\t}"
+      : "=f"(r) : "f"(m), "f"(a), "f"(b));
+  return r;
+}
+
 // B operand of a run of 32 inputs (two k-steps): pairs (x_i, x_{i+4}), i < 4, of
 // this thread's eight inputs, split into three BF16 parts.
 struct BRun {
   uint32_t hi[4], mid[4], lo[4];
 };
 
-// Returns whether the three parts of each input are the input. They are from 2^-110
-// on; below, an input may have bits under 2^-133, which BF16 has not, and an infinity
-// or NaN leaves a NaN: either way what is left of the third part has low bits.
-__device__ __forceinline__ bool split_run(const float4& xa, const float4& xb, BRun& b) {
+// What tells whether the MMAs can take a thread's inputs of a group: each is below
+// 2^113 (128 of them times codes then sum to less than 2^123) and its three parts are
+// the input. They are from 2^-110 on; below, an input may have bits under 2^-133, which
+// BF16 has not, and an infinity or NaN leaves a NaN: either way what is left of the
+// third part has low bits.
+struct XRange {
+  float most;
+  uint32_t left;
+  __device__ bool ok() const { return (left & 0xFFFFu) == 0u && most < 0x1p113f; }
+};
+
+__device__ __forceinline__ void split_run(const float4& xa, const float4& xb, BRun& b, XRange& xr) {
   const float a[4] = {xa.x, xa.y, xa.z, xa.w}, c[4] = {xb.x, xb.y, xb.z, xb.w};
-  uint32_t left = 0u;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
+    xr.most = max3_abs(xr.most, a[i], c[i]);
     b.hi[i] = upper_pair(a[i], c[i]);
     const float2 r = __fadd2_rn(make_float2(a[i], c[i]), make_float2(-upper(a[i]), -upper(c[i])));
     b.mid[i] = upper_pair(r.x, r.y);
     const float2 s = __fadd2_rn(r, make_float2(-upper(r.x), -upper(r.y)));
     b.lo[i] = upper_pair(s.x, s.y);
-    left |= __float_as_uint(s.x) | __float_as_uint(s.y);
+    xr.left |= __float_as_uint(s.x) | __float_as_uint(s.y);
   }
-  return (left & 0xFFFFu) == 0u;
 }
 
 // Codes i and i + 4 of a code word as a BF16 pair: 128 + u (u = code + 8) in the
@@ -250,8 +266,10 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
       for (int t = 0; t < NT; ++t) ec[r][t] = e[r][t];
     }
     if (gr + 1 < g1) load(gr + 1);
+    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     float rh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     TileRec tr[2];
+    XRange xr{0.0f, 0u};
     bool any = false;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -275,47 +293,64 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
         for (int r = 0; r < 2; ++r) nb[r] = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + win);
       }
       BRun b;
-      // Vectors that the MMAs cannot take in this run: inputs too small for the split, or
-      // an infinity or NaN (a row whose A is zero there, with no record or in another
-      // tile's lanes, would get 0 * infinity)
-      const unsigned odd = __ballot_sync(0xffffffffu, !split_run(xa, xb, b));
-      const float* xr = tk.x + 128 * gr + 32 * j + 8 * q;
-      if (odd && ((odd >> (lane & 28)) & 15u) != 0u) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) b.hi[i] = b.mid[i] = b.lo[i] = 0u;
-      }
+      split_run(xa, xb, b, xr);
       uint32_t c0[4], c1[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         c0[i] = code_pair(wc[0][j], i);
         c1[i] = code_pair(wc[1][j], i);
       }
-      if (odd) {
-        float o[4];
-        run_fp32(xr, tk.cols, odd, q, c0, c1, true, true, o);
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (sc[i >> 1] != 0.0f) acc[i] = __fmaf_rn(o[i], sc[i >> 1], acc[i]);
-      }
-      float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
       mma_run(h, ml, c0, c1, b);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)  // an all-zero group (scale 0) adds nothing, whatever x holds
-        if (sc[i >> 1] != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sc[i >> 1], acc[i]);
       if (any) {
         residual_pairs(tr[0], nb[0], c0);
         residual_pairs(tr[1], nb[1], c1);
-        if (odd) {
-          float o[4];
-          run_fp32(xr, tk.cols, odd, q, c0, c1, ec[0][t] != 0ull, ec[1][t] != 0ull, o);
-#pragma unroll
-          for (int i = 0; i < 4; ++i) racc[i] = __fadd_rn(racc[i], o[i]);
-        }
         mma_run(rh, rml, c0, c1, b);
       }
     }
+    // Vectors that the MMAs could not take (inputs too small for the split, too large for
+    // the sums, an infinity or NaN) get the group again on the FP32 pipes. Their columns
+    // of the accumulators are their own.
+    const unsigned odd = __ballot_sync(0xffffffffu, !xr.ok());
+    if (odd) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
+      for (int i = 0; i < 4; ++i)
+        if ((odd >> (8 * q + 4 * (i & 1))) & 15u) h[i] = ml[i] = rh[i] = rml[i] = 0.0f;
+#pragma unroll 1
+      for (int j = 0; j < 4; ++j) {
+        const float* xj = tk.x + 128 * gr + 32 * j + 8 * q;
+        uint32_t c0[4], c1[4];
+        float o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          c0[i] = code_pair(__ldg(cp[0] + 16 * gr + 4 * j), i);
+          c1[i] = code_pair(__ldg(cp[1] + 16 * gr + 4 * j), i);
+        }
+        run_fp32(xj, tk.cols, odd, q, c0, c1, true, true, o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (sc[i >> 1] != 0.0f) acc[i] = __fmaf_rn(o[i], sc[i >> 1], acc[i]);
+        if (!mp[0]) continue;
+        unsigned long long en[2];
+        const int jt = 32 * j + 8 * q;  // the thread's first input in the group
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          en[r] = __ldg(mp[r] + ((128 * gr + jt) >> LC));
+          tr[r] = tile_rec<LC>(a, en[r]);
+          const uint4 nb = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + ((jt & ((1 << LC) - 1)) >> 3));
+          residual_pairs(tr[r], nb, r ? c1 : c0);
+        }
+        run_fp32(xj, tk.cols, odd, q, c0, c1, en[0] != 0ull, en[1] != 0ull, o);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) racc[i] = __fadd_rn(racc[i], o[i]);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      // an all-zero group (scale 0) adds nothing, whatever x holds
+      const float sr = sc[i >> 1];
+      if (sr != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sr, acc[i]);
+      racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
+    }
   }
   // c = 2^-(LC/2) is folded into the residual for C = 64 and 16; C = 32 had 1/8
   const float cf = LC == 5 ? __fmul_rn(8.0f, pr.c) : 1.0f;
