@@ -26,12 +26,13 @@
 // (lane / 4, lane % 4) takes inputs 8q .. 8q + 7, one code word of rows g and g + 8, one
 // nibble-table window, two float4 of vector g.
 //
-// A warp takes 16 rows and a slice of the columns; slices of a row tile sit in one
-// block and are summed through shared memory in a fixed order, so a product's bits do
-// not depend on what shares its launch.
+// A warp takes 16 rows and a slice of the columns. A row tile's product is always made
+// of the same eight column sums, added in order through the shared memory of the block
+// that has all its slices: how many slices there are (one to eight) depends on what
+// else is in the launch, the product's bits do not.
 //
 // One 3B-shaped layer (77 M weights, 0.162 bits/weight of records, SDQ scales, eight
-// vectors, one batched launch): 263 -> 66 us on the device, 308 -> 76 us a call. Its
+// vectors, one batched launch): 308 -> 79 us a call. Its
 // relative error against 64 bits is 9.6e-8 where the FP32 pipes' sums had 1.4e-7.
 // Bound by issue (46% of slots): 370 instructions per 16 rows and 128 inputs for the
 // backbone (half of them the split of x) and up to 380 for the residual.
@@ -45,6 +46,7 @@ namespace awsrc {
 namespace {
 
 constexpr int kWarps = 8;
+constexpr int kSums = 8;  // column slices whose sums make up a row tile's
 
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
@@ -206,7 +208,7 @@ __device__ __forceinline__ void run_fp32(const float* x, int64_t cols, unsigned 
 
 template <int LC>
 __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const __grid_constant__ GemvArgs a, int M) {
-  __shared__ float4 part[kWarps][32];
+  __shared__ float4 part[kWarps][kSums][32];  // [row tile of the block][sum][lane]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
   int ti = 0;
   for (int i = 1; i < a.n_task; ++i)
@@ -215,7 +217,12 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
   const int ks = tk.slices, slice = warp & (ks - 1), per = kWarps / ks;  // slices: a power of two up to kWarps
   const int64_t row0 = ((int64_t)(blockIdx.x - tk.block0) * per + warp / ks) * 16;
   const int gpr = (int)(tk.cols >> 7);
-  const int g0 = gpr * slice / ks, g1 = row0 < tk.rows ? gpr * (slice + 1) / ks : g0;
+  // the warp's groups: kSums / ks of the row tile's eight sums (some empty when gpr < 8)
+  auto bound = [gpr](int i) { return (int)((int64_t)gpr * i / kSums); };
+  int sum = kSums / ks * slice;
+  const int g0 = bound(sum), g1 = row0 < tk.rows ? bound(sum + kSums / ks) : g0;
+  while (sum < kSums - 1 && bound(sum + 1) <= g0) ++sum;  // the sum that holds group g0
+  int sum_end = bound(sum + 1);
   int64_t row[2];
 #pragma unroll
   for (int r = 0; r < 2; ++r) row[r] = min(row0 + g + 8 * r, tk.rows - 1);  // rows past the end repeat the last one
@@ -252,6 +259,8 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
         e[r][t] = mp[r] ? __ldg(mp[r] + (LC >= 5 ? NT * gr + t : 8 * gr + 2 * t + (q >> 1))) : 0ull;
     }
   };
+  // c = 2^-(LC/2) is folded into the residual for C = 64 and 16; C = 32 had 1/8
+  const float cf = LC == 5 ? __fmul_rn(8.0f, pr.c) : 1.0f;
   float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, racc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   if (g0 < g1) load(g0);
   for (int gr = g0; gr < g1; ++gr) {
@@ -351,23 +360,27 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
       if (sr != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sr, acc[i]);
       racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
     }
-  }
-  // c = 2^-(LC/2) is folded into the residual for C = 64 and 16; C = 32 had 1/8
-  const float cf = LC == 5 ? __fmul_rn(8.0f, pr.c) : 1.0f;
-  float v[4];
+    if (gr + 1 == sum_end) {
+      float v[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) v[i] = __fmaf_rn(racc[i], cf, acc[i]);
-  if (ks > 1) {
-    part[warp][lane] = make_float4(v[0], v[1], v[2], v[3]);
-    __syncthreads();
-    if (slice == 0) {
-      for (int i = 1; i < ks; ++i) {
-        const float4 p = part[warp + i][lane];
-        v[0] = __fadd_rn(v[0], p.x);
-        v[1] = __fadd_rn(v[1], p.y);
-        v[2] = __fadd_rn(v[2], p.z);
-        v[3] = __fadd_rn(v[3], p.w);
+      for (int i = 0; i < 4; ++i) {
+        v[i] = __fmaf_rn(racc[i], cf, acc[i]);
+        acc[i] = racc[i] = 0.0f;
       }
+      part[warp / ks][sum][lane] = make_float4(v[0], v[1], v[2], v[3]);
+      while (sum < kSums - 1 && sum_end <= gr + 1) sum_end = bound(++sum + 1);
+    }
+  }
+  __syncthreads();
+  float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  if (slice == 0 && row0 < tk.rows) {
+    for (int i = 0; i < kSums; ++i) {
+      if (bound(i) == bound(i + 1)) continue;
+      const float4 p = part[warp / ks][i][lane];
+      v[0] = __fadd_rn(v[0], p.x);
+      v[1] = __fadd_rn(v[1], p.y);
+      v[2] = __fadd_rn(v[2], p.z);
+      v[3] = __fadd_rn(v[3], p.w);
     }
   }
   if (slice == 0) {
@@ -391,24 +404,40 @@ bool gemv_mma(const Prm& pr, const GemvArgs& a, int M) {
 
 cudaError_t launch_gemv_mma(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st) {
   GemvArgs b = a;
-  // slices of about eight groups (4, 8, 12 and 16 groups measured 70, 66, 66 and 78 us
-  // on the layer above): the shape alone decides, so that a product's sums are the
-  // same in every batch
-  auto slices = [](const GemvTask& t) {
-    const int64_t gpr = t.cols >> 7;
-    int s = 1;
-    while (s < kWarps && gpr > 8 * s) s <<= 1;
-    return s;
-  };
+  int dev = 0, nsm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  // Slices of at most eight groups (of four: 84 us instead of 77 on the layer above), and
+  // shorter ones while the launch has less than 1.75 waves of warps: a warp takes 2 to
+  // 3.4 us per group however empty the chip is, so a 2048 x 2048 module alone went from
+  // 29 us (two slices) to 10 (eight), an 11008 x 2048 one from 35 to 29, a gate and up pair
+  // (now four slices) from 59 to 52.
+  int64_t warps = 0;
+  auto tiles = [](const GemvTask& t) { return (t.rows + 15) / 16; };
+  auto groups = [](const GemvTask& t) { return ((t.cols >> 7) + t.slices - 1) / t.slices; };  // of a slice
+  for (int i = 0; i < b.n_task; ++i) {
+    GemvTask& t = b.t[i];
+    t.slices = 1;
+    while (t.slices < kWarps && groups(t) > 8) t.slices <<= 1;
+    warps += tiles(t) * t.slices;
+  }
+  while (warps < (int64_t)nsm * 2 * kWarps * 7 / 4) {
+    GemvTask* m = nullptr;  // the task with the longest slices
+    for (int i = 0; i < b.n_task; ++i) {
+      GemvTask& t = b.t[i];
+      if (t.slices < kWarps && groups(t) > 1 && (!m || groups(t) > groups(*m))) m = &t;
+    }
+    if (!m) break;
+    warps += tiles(*m) * m->slices;
+    m->slices <<= 1;
+  }
   // the tasks with the longest slices first, so that their blocks do not end the
   // launch (69 us in the caller's order, the down projection last)
-  std::stable_sort(b.t, b.t + b.n_task, [&](const GemvTask& x, const GemvTask& y) {
-    return (x.cols >> 7) * slices(y) > (y.cols >> 7) * slices(x);
-  });
+  std::stable_sort(b.t, b.t + b.n_task, [&](const GemvTask& x, const GemvTask& y) { return groups(x) > groups(y); });
   int64_t blocks = 0;
   for (int i = 0; i < b.n_task; ++i) {
     GemvTask& t = b.t[i];
-    t.slices = slices(t);
     const int64_t per = 16 * (kWarps / t.slices);
     t.block0 = (int)blocks;
     blocks += (t.rows + per - 1) / per;

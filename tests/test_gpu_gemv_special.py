@@ -121,3 +121,18 @@ def test_largest_record_scale(orc, C):
     want, yabs = definition(x)
     assert np.isfinite(gemv(x[:1])).all() and np.abs(want).max() > 2.0 ** 80
     assert (np.abs(y - want) <= _bound(cols, C, yabs)).all()
+
+
+@pytest.mark.parametrize("cols", [128, 384, 1152, 2048, 2432])
+def test_bits_do_not_depend_on_the_batch(cols):
+    """A product beside a task that fills the chip (fewer, longer column slices) has the
+    bits of its single call (eight slices)."""
+    import paper_2608_23144_gb300 as aw
+    rng = np.random.default_rng(91)
+    shapes, M = [(70000, 128), (50, cols)], 8
+    prm = aw.params(C=64, P=4, b=4, S=64)
+    bbs = [aw.awsrc_rtn_quantize(torch.from_numpy(rng.normal(0, 0.02, s).astype(np.float32)).cuda()) for s in shapes]
+    xs = [torch.from_numpy(rng.normal(0, 1, (M, s[1])).astype(np.float32)).cuda() for s in shapes]
+    both = aw.awsrc_packed_gemv_batch(prm, shapes, [(0, bbs[0], xs[0]), (1, bbs[1], xs[1])])
+    for m in (0, 1):
+        assert torch.equal(both[m], aw.awsrc_packed_gemv(prm, shapes, m, bbs[m], xs[m]))
