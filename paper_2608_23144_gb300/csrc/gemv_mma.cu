@@ -395,11 +395,30 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
 
 }  // namespace
 
-// From three vectors on: the layer of the figures above takes 65 us here whatever
-// M is, against 30, 47, 125 and 263 us for M = 1, 2, 3 and 8 on the FP32 pipes.
-bool gemv_mma(const Prm& pr, const GemvArgs& a, int M) {
+// From three vectors on, where the tensor cores are estimated to be faster on the
+// module list. The list decides, and M, not the tasks of a call: a product's bits are
+// the same in every call on the list. In us, fitted to single modules and whole layers
+// of 0.03 to 275 M weights, M = 3 to 8 (records at 0.162 bits/weight; without records
+// both sides take about 0.6 of it):
+//  * here 3 + the larger of 0.4 per group of the widest module (a warp's slice, an
+//    eighth of them, one group after the other) and 1.05 per million weights, whatever M;
+//  * on the FP32 pipes 3 + (0.3 + 0.21 M) per million weights, and M where the inputs do
+//    not fit in shared memory (gemv.cu).
+// Measured, FP32 pipes against tensor cores: 1024 x 1024, M = 4: 4.6 and 6.3; 2048 x
+// 2048, M = 3 and 8: 8.0 and 9.9, 14.2 and 10.2; 512 x 11008, M = 4 and 8: 20.3 and 37.7,
+// 38.4 and 38.8; 11008 x 2048, M = 3 and 5: 24.4 and 28.7, 33.0 and 29.2; the layer above,
+// M = 3 and 8: 125 and 77, 267 and 78.
+bool gemv_mma(const Prm& pr, const GemvArgs& a, int M, int n_mod, const awsrc_module* mods) {
   const bool c = pr.C == 16 || pr.C == 32 || pr.C == 64;
-  return M >= 3 && c && (!a.map || (a.nib && pr.scale_mode == AWSRC_SCALE_POW2));
+  if (M < 3 || !c || (a.map && (!a.nib || pr.scale_mode != AWSRC_SCALE_POW2))) return false;
+  double widest = 0.0, weights = 0.0, fp32 = 0.0;
+  for (int m = 0; m < n_mod; ++m) {
+    const double w = 1e-6 * (double)mods[m].rows * (double)mods[m].cols;
+    weights += w;
+    widest = std::max(widest, (double)(mods[m].cols >> 7));
+    fp32 += w * (gemv_in_smem(mods[m].cols, M) ? 0.3 + 0.21 * M : (double)M);
+  }
+  return fp32 >= std::max(0.4 * widest, 1.05 * weights);
 }
 
 cudaError_t launch_gemv_mma(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st) {
