@@ -328,6 +328,11 @@ awsrc_status awsrc_select_workspace_bytes(const awsrc_params* prm, int32_t n_mod
  *      d_bytes[r] = h + K_r*L.
  *   stream_out  device, >= awsrc_stream_capacity() bytes: header + records.
  *   d_counts, d_bytes  device int64 arrays as above.
+ * One kernel whose blocks meet at grid barriers, launched cooperatively: it
+ * starts when all its blocks fit on the device at once, beside whatever other
+ * streams run there. The barriers' waits are bounded (2 s each); should one give
+ * up, awsrc_workspace_status(workspace) reports bit 2, and stream_out, d_counts
+ * and d_bytes are undefined (never past their ends).
  * Stream layout (little-endian): header of 40 + 8*n_mod bytes, then fixed-width
  * records of L bytes. Record bits are LSB-first from bit 0: tile (ceil(log2 T)
  * bits), seed (ceil(log2 S)), scale field (b_e), codes 0..P-1 (b bits each, two's
@@ -530,17 +535,18 @@ void awsrc_set_search_pruning(int32_t enabled);
  * awsrc_set_wait_test — a test of the kernels' failure handling, for the
  * calling host thread (no counterpart in the paper). Every wait inside the
  * tcgen05 search kernels (for bulk copies, tensor-core results and the release
- * of shared buffers) gives up after a time limit, 2 s by default; the block
- * then records bit 2 of the workspace's fault word, waits (with the same
- * limit) for its own copies and tensor-core work still in flight, frees its
- * tensor memory and exits, so the GPU context stays usable.
- *   wait_ns      the limit of every such wait in later awsrc_encode_tiles
- *                calls (0: the default 2 s).
+ * of shared buffers) and at the selection kernel's grid barriers gives up after
+ * a time limit, 2 s by default; the block then records bit 2 of the workspace's
+ * fault word, waits (with the same limit) for its own copies and tensor-core
+ * work still in flight, frees its tensor memory and exits (at a barrier: every
+ * block leaves), so the GPU context stays usable.
+ *   wait_ns      the limit of every such wait in later awsrc_encode_tiles and
+ *                awsrc_select_records calls (0: the default 2 s).
  *   stall_chunk  >= 0: the C = 64, P = 4, AWSRC-U search issues no copies of
  *                its seed chunks from this one (counted within each block's
  *                range of 32-seed chunks) on, so its waits for that chunk run
  *                out; -1: normal operation.
- * The call's candidates are then undefined and awsrc_workspace_status reports
+ * The call's outputs are then undefined and awsrc_workspace_status reports
  * bit 2. awsrc_set_wait_test(0, -1) restores normal operation.
  */
 void awsrc_set_wait_test(uint64_t wait_ns, int32_t stall_chunk);

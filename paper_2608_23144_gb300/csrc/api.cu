@@ -599,6 +599,7 @@ awsrc_status awsrc_select_records(const awsrc_params* prm, int32_t n_mod, const 
   SelectPlan sp;
   std::vector<int64_t> to, kc;
   if ((s = select_plan(pr, n_mod, mods, rates_bpw, n_rates, &sp, &to, &kc)) != AWSRC_OK) return s;
+  if (g_wait_ns) pr.wait_ns = g_wait_ns;
   if (!cands || !stream_out || !d_counts || !d_bytes) return AWSRC_ERR_INVALID_ARG;
   if (!aligned(cands, 4) || !aligned(d_counts, 8) || !aligned(d_bytes, 8)) return AWSRC_ERR_INVALID_ARG;
   if (stream_capacity < (size_t)(sp.h + sp.cap_records * sp.L)) return AWSRC_ERR_CAPACITY;

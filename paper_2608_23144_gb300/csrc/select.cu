@@ -85,6 +85,7 @@ __device__ __forceinline__ uint32_t gain_field(float g) {
 struct GridBarrier {
   unsigned* bar;
   unsigned phase;
+  uint64_t limit_ns;
   __device__ bool sync() {
     __syncthreads();
     bool ok = true;
@@ -97,7 +98,7 @@ struct GridBarrier {
       if (vb[0] < target) {
         const uint64_t t0 = tc05::globaltimer();
         while (vb[0] < target) {
-          if (vb[1] != 0u || tc05::globaltimer() - t0 > kWaitLimitNs) {
+          if (vb[1] != 0u || tc05::globaltimer() - t0 > limit_ns) {
             atomicExch(bar + 1, 1u);
             ok = false;
             break;
@@ -327,7 +328,7 @@ __global__ void __launch_bounds__(ST, 2) select_kernel(const awsrc_candidate* __
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool pf = a.variant != AWSRC_VARIANT_U;
   const int nseg = pf ? 1 : a.n_mod;
-  GridBarrier bar{w.bar, 0u};
+  GridBarrier bar{w.bar, 0u, pr.wait_ns};
   // tiles of this block, and of segment m
   const int64_t per = (a.T + gridDim.x - 1) / gridDim.x;
   const int64_t t0 = min(a.T, (int64_t)blockIdx.x * per), t1 = min(a.T, t0 + per);
