@@ -542,10 +542,10 @@ void awsrc_set_search_pruning(int32_t enabled);
  * block leaves), so the GPU context stays usable.
  *   wait_ns      the limit of every such wait in later awsrc_encode_tiles and
  *                awsrc_select_records calls (0: the default 2 s).
- *   stall_chunk  >= 0: the C = 64, P = 4, AWSRC-U search issues no copies of
- *                its seed chunks from this one (counted within each block's
- *                range of 32-seed chunks) on, so its waits for that chunk run
- *                out; -1: normal operation.
+ *   stall_chunk  >= 0: the C = 64, P = 4 searches issue no copies of their
+ *                seed chunks from this one (counted within each block's range
+ *                of 32-seed chunks, AWSRC-P_F: 12-seed chunks) on, so their
+ *                waits for that chunk run out; -1: normal operation.
  * The call's outputs are then undefined and awsrc_workspace_status reports
  * bit 2. awsrc_set_wait_test(0, -1) restores normal operation.
  */

@@ -780,7 +780,7 @@ def awsrc_set_search_pruning(enabled: bool):
 def awsrc_set_wait_test(wait_ns: int = 0, stall_chunk: int = -1):
     """For this host thread: the limit of the encoder's and the selection's
     bounded waits (0 = 2 s) and, for stall_chunk >= 0, the seed chunk from which
-    the C = 64, P = 4 U search issues no copies, so that its waits run out (a
+    the C = 64, P = 4 searches issue no copies, so that their waits run out (a
     test of the timeout path). awsrc_set_wait_test() restores normal operation."""
     lib.awsrc_set_wait_test(int(wait_ns), int(stall_chunk))
 

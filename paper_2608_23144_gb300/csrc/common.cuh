@@ -43,8 +43,8 @@ struct Prm {
   int fast_pow2;  // POW2 scale whose exponent range can never bind for a valid candidate
   uint32_t mant_q;  // mantissa field of (float)qmax
   int prune;        // 1: the C = 64, P = 4 U search skips candidates its bound rules out
-  int stall_chunk;  // test of the bounded waits: the U search's producer issues no copies from
-                    // this chunk of its block's range on (-1: never)
+  int stall_chunk;  // test of the bounded waits: the tcgen05 searches issue no copies from this
+                    // chunk of a block's range on (-1: never)
   uint64_t wait_ns; // limit of every bounded wait inside a kernel (2 s)
 };
 

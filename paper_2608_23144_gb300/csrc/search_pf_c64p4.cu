@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(NT, 1)
     ++issued;
   };
   if (warp == EW + 1 && lane == 0)
-    while (issued < STAGES && issued < nck) load_chunk();
+    while (issued < STAGES && issued < nck && issued != pr.stall_chunk) load_chunk();
   // stage y = d * r and d, d = w_act * a + w_fisher * F (per element)
   for (int e = tid; e < BM * 64; e += NT) {
     const int r = e >> 6, j = e & 63;
@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(NT, 1)
   } else if (warp == EW + 1) {
     // --------------------------------------------------------------- loader --
     if (lane == 0) {
-      while (issued < nck) {  // the stage of chunk issued - STAGES, once its MMAs are complete
+      while (issued < nck && issued != pr.stall_chunk) {  // the stage of chunk issued - STAGES, once its MMAs are complete
         if (!mbar_wait(&sm.sfree[issued % STAGES], (uint32_t)((issued / STAGES - 1) & 1), pr.wait_ns)) { timed_out = true; break; }
         load_chunk();
       }
@@ -605,7 +605,8 @@ __global__ void __launch_bounds__(NT, 1)
         bsd = (uint32_t)(sx + (g2[0].x == cm ? 0 : g2[0].y == cm ? 1 : g2[1].x == cm ? 2 : 3));
       }
     }
-    sm.red_g[grp][m] = unit ? __fmul_rn(-bg, sm.from_unit[m]) : -bg;
+    // (a loss of +0 is a gain of +0, not -0)
+    sm.red_g[grp][m] = unit ? __fadd_rn(0.0f, __fmul_rn(-bg, sm.from_unit[m])) : -bg;
     sm.red_s[grp][m] = bsd;
   }
   tc_fence_before();
