@@ -28,6 +28,7 @@
 // every key in 16 to 20 launches per call took 160 and 901 us.
 #include <algorithm>
 #include <cfloat>
+#include <cuda.h>
 
 #include "internal.h"
 #include "tc05.cuh"
@@ -745,6 +746,29 @@ SelLayout select_layout(const SelectPlan& sp, bool pf) {
   return l;
 }
 
+// SMs that kernels of stream `st` may use, of the device's nsm: fewer in a green
+// context. A cooperative launch is checked against the device's count only, and
+// blocks beyond what the stream's SMs hold would never meet the others at a barrier.
+int stream_sms(cudaStream_t st, int nsm) {
+  using GetCtx = CUresult (*)(CUstream, CUcontext*, CUgreenCtx*);
+  using GetRes = CUresult (*)(CUgreenCtx, CUdevResource*, CUdevResourceType);
+  auto entry = [](const char* name, unsigned version) {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &found);
+    return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? f : nullptr;
+  };
+  static const GetCtx get_ctx = reinterpret_cast<GetCtx>(entry("cuStreamGetCtx", 12050));
+  static const GetRes get_res = reinterpret_cast<GetRes>(entry("cuGreenCtxGetDevResource", 12040));
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  CUdevResource r;
+  if (!get_ctx || !get_res || get_ctx(st, &ctx, &green) != CUDA_SUCCESS || !green ||
+      get_res(green, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS)
+    return nsm;
+  return std::max(1, std::min(nsm, (int)r.sm.smCount));
+}
+
 }  // namespace
 
 size_t select_ws_bytes(const Prm& pr, const SelectPlan& sp) {
@@ -795,7 +819,7 @@ awsrc_status select_run(const Prm& pr, const SelectPlan& sp, const int64_t* tile
   // as many blocks as are resident at once, fewer when a block would get less
   // than two rounds of tiles (a barrier costs more, the more blocks meet at it)
   const int64_t want = (sp.T + 4 * ST - 1) / (4 * ST);
-  const int64_t grid = std::max<int64_t>(1, std::min({want, (int64_t)nsm * per_sm, kMaxBlocks}));
+  const int64_t grid = std::max<int64_t>(1, std::min({want, (int64_t)stream_sms(st, nsm) * per_sm, kMaxBlocks}));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(ST);
