@@ -70,7 +70,8 @@ template <> struct Elt<__nv_bfloat16> {
 
 constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23: x + kMagic rounds x to an integer (ties to even)
 
-// Codes of two inputs for a normal binary16 s, rs = RN(1/s). t = RN(w rs) =
+// Codes of two inputs for a normal binary16 s, rs = RN(1/s). t = RN(w rs), or w rs
+// itself where the product is contracted into the sums below, is
 // (w / s)(1 + d) with |d| < 2^-23 + 2^-48 and |w / s| <= 7.004, so
 // |t - RN(w / s)| < 2^-20 and rint(t) = rint(RN(w / s)) unless t is within
 // 2^-20 of a half-integer; `tie` is set when |t - rint(t)| > 1/2 - 2^-16 (the

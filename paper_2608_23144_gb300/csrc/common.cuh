@@ -4,8 +4,10 @@
 //
 // Every floating-point operation that decides an integer output is written
 // with an explicit round-to-nearest intrinsic (__fmaf_rn, __fmul_rn, ...), and
-// the library is compiled with --fmad=false, so the compiler cannot fuse or
-// reorder them: the order is the one the public header fixes.
+// the library is compiled with --fmad=false, so the compiler does not fuse or
+// reorder them: the order is the one the public header fixes. One pair escapes
+// that: __fmul2_rn feeding __fadd2_rn becomes a packed fma. Where such a product is
+// not exact, the addition is written with scalars.
 #pragma once
 
 #include <cstdint>

@@ -203,6 +203,24 @@ template <> struct Io2<__nv_bfloat16> {
   }
 };
 
+// o = w + r with r rounded first. A packed multiplication that feeds a packed addition
+// is contracted to one fused operation, which is the same only where the product is
+// exact: a power of two times k_j c, c a power of two. Elsewhere (C = 32 or binary16
+// scales, where fused sums were off by a bit) the additions are scalar.
+template <typename TI, typename TO, int G>
+__device__ __forceinline__ void add_rounded(const Prm& pr, const Vec<TI, G>& w, const float2* r, Vec<TO, G>& o) {
+  if (pr.scale_mode == AWSRC_SCALE_POW2 && (pr.logC & 1) == 0) {
+#pragma unroll
+    for (int e = 0; e < G; e += 2) Io2<TO>::st(o.v + e, __fadd2_rn(Io2<TI>::ld(w.v + e), r[e / 2]));
+  } else {
+#pragma unroll
+    for (int e = 0; e < G; e += 2) {
+      const float2 v = Io2<TI>::ld(w.v + e);
+      Io2<TO>::st(o.v + e, make_float2(__fadd_rn(v.x, r[e / 2].x), __fadd_rn(v.y, r[e / 2].y)));
+    }
+  }
+}
+
 // One G-element vector of a recorded tile: o_j = fl(w_j + fl(fl(k_j * c) * sc))
 // with k_j = sum_p sign_{j,p} * code_p = tot - 2 * sum_p bit_{j,p} * code_p
 // (exact integers); mk points at atom 0's mask word of the vector, j0 its first
@@ -225,12 +243,13 @@ __device__ __forceinline__ void patch_vec(const Prm& pr, const Vec<TI, G>& w, ui
     }
   }
   const float2 c2 = make_float2(pr.c, pr.c), s2 = make_float2(sc, sc);
+  float2 r[G / 2];
 #pragma unroll
   for (int e = 0; e < G; e += 2) {
     const float2 k = make_float2((float)(tot - 2 * acc[e]), (float)(tot - 2 * acc[e + 1]));
-    const float2 r = __fmul2_rn(__fmul2_rn(k, c2), s2);
-    Io2<TO>::st(o.v + e, __fadd2_rn(Io2<TI>::ld(w.v + e), r));
+    r[e / 2] = __fmul2_rn(__fmul2_rn(k, c2), s2);
   }
+  add_rounded<TI, TO, G>(pr, w, r, o);
 }
 
 // The record slot of the dense decoder: the codes (x, y; code p in byte p)
@@ -269,11 +288,12 @@ __device__ __forceinline__ void patch_vec_tab(const Prm& pr, const Vec<TI, G>& w
     for (int e = 0; e < G; ++e) k[e] = __fmul_rn(k[e], pr.c);
   }
   const float2 s2 = make_float2(sc, sc);
+  float2 r[G / 2];
 #pragma unroll
   for (int e = 0; e < G; e += 2) {
-    const float2 r = __fmul2_rn(make_float2(k[e], k[e + 1]), s2);
-    Io2<TO>::st(o.v + e, __fadd2_rn(Io2<TI>::ld(w.v + e), r));
+    r[e / 2] = __fmul2_rn(make_float2(k[e], k[e + 1]), s2);
   }
+  add_rounded<TI, TO, G>(pr, w, r, o);
 }
 
 // Dense-mode record pass: record k's slot (record_slot) goes to codes[k] and
