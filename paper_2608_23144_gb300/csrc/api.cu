@@ -19,7 +19,8 @@ thread_local int g_prune = 1;
 thread_local uint64_t g_wait_ns = 0;  // 0: the default limit
 thread_local int g_stall_chunk = -1;
 std::atomic<uint64_t> g_launches{0};
-constexpr int64_t kTargetBlocks = 1216;  // enough blocks to fill a GB300 (152 SMs) several times
+constexpr int kSms = 152;                // of a GB300
+constexpr int64_t kTargetBlocks = 8 * kSms;  // enough blocks to fill it several times
 // one RTN launch has a block per 256 groups of 128 weights: 2^46 weights keep
 // its grid far inside gridDim.x and every size product inside int64
 constexpr int64_t kMaxBackboneWeights = 1ll << 46;
@@ -86,6 +87,32 @@ struct EncodeLayout {
   bool mma;      // mma.sync search
 };
 
+// Seed splits of the mma.sync search for `base` runs of tiles and `units` groups of
+// seeds, with `slots` blocks resident at once. Enough splits for kTargetBlocks, as the
+// other searches have them, are right for large calls; in small ones they left an item
+// one or two groups of seeds and the merge a hundred candidates of every tile (1024
+// tiles of 16, S = 1024, P = 2: 56 us in 128 splits, 26 in 38), where too few leave a
+// wave nearly empty (8192 tiles, S = 4096: 150 us in 19 splits, 198 in 5). So calls of at
+// most one run per slot take the least of, in groups, waves x (an item's groups + 4) + a
+// fifth per split, if that is 10% less; a last wave that is filled to less than a third
+// counts as 0.6. (Not where an SM holds one block, P_F with C = 64 and 128: its groups
+// are dear, and fewer splits cost up to 20%.)
+int64_t mma_splits(int64_t base, int64_t units, int64_t slots) {
+  const int64_t most = std::max<int64_t>(1, std::min((kTargetBlocks + base - 1) / base, units));
+  if (base > slots || slots <= kSms) return most;
+  auto cost = [&](int64_t ns) {
+    const int64_t items = ns * base, full = items / slots, rest = items % slots;
+    const int64_t tenths = 10 * full + (rest == 0 ? 0 : full > 0 && 10 * rest <= 3 * slots ? 6 : 10);
+    return tenths * ((units + ns - 1) / ns + 4) + 2 * ns;
+  };
+  int64_t best = most;
+  for (int64_t ns = 1; ns < most; ++ns) {
+    const int64_t per = (units + ns - 1) / ns;
+    if ((units + per - 1) / per == ns && cost(ns) < cost(best)) best = ns;  // (no empty splits)
+  }
+  return 10 * cost(best) <= 9 * cost(most) ? best : most;
+}
+
 EncodeLayout encode_layout(const Prm& pr, int32_t n_mod, const awsrc_module* mods, int64_t T) {
   EncodeLayout L{};
   L.spec = use_c64p4(pr);
@@ -104,7 +131,7 @@ EncodeLayout encode_layout(const Prm& pr, int32_t n_mod, const awsrc_module* mod
                        : L.spec_pf ? pr.S_pad / search_pf_c64p4_chunk()
                        : L.mma     ? (pr.S + 7) / 8  // groups of eight seeds
                                    : (pr.S + gs.lanes - 1) / gs.lanes;
-  int64_t ns = (kTargetBlocks + base_blocks - 1) / base_blocks;
+  int64_t ns = L.mma ? mma_splits(base_blocks, units, search_mma_slots(pr)) : (kTargetBlocks + base_blocks - 1) / base_blocks;
   ns = std::max<int64_t>(1, std::min<int64_t>(ns, units));
   L.nsplit = (int)ns;
   size_t off = kStatusBytes;

@@ -78,6 +78,7 @@ cudaError_t launch_search_generic(const Prm& pr, const LaunchDesc& ld, const uin
 // P in {2, 4} (search_mma.cuh) in items of search_mma_tiles() consecutive tiles
 // and one seed split; same candidate output. `pairs`: the paired Gram table.
 int search_mma_tiles();
+int search_mma_slots(const Prm& pr);  // blocks that a GB300 holds at once (with BF16 weights)
 cudaError_t launch_search_mma_u(const Prm& pr, const LaunchDesc& ld, const uint64_t* masks, const float2* pairs,
                                 int64_t n_items, awsrc_candidate* cands, cudaStream_t st);
 cudaError_t launch_search_mma_pf(const Prm& pr, const LaunchDesc& ld, const uint64_t* masks, int64_t n_items,

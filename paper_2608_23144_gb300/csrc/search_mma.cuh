@@ -59,6 +59,9 @@ __host__ __device__ constexpr int mma_groups(int P, int VAR, int KS) {
   return n < 1 ? 1 : n;
 }
 
+// blocks per SM that the registers allow
+__host__ __device__ constexpr int mma_per_sm(int VAR, int KS) { return VAR == AWSRC_VARIANT_PF && KS >= 4 ? 1 : 2; }
+
 __device__ __forceinline__ float ninf() { return -__int_as_float(0x7f800000); }
 
 // D += A B on m16n8k16 (FP16 operands, binary32 accumulation).
@@ -438,7 +441,7 @@ __device__ __forceinline__ void mma_build_table(const Prm& pr, const uint64_t* _
 // BF: W and W0 of every module are BF16 and copied ahead (kLoadAsync), known at
 // compile time.
 template <int P, int VAR, int KS, bool FAST, bool BF>
-__global__ void __launch_bounds__(32 * kMmaWarps, (VAR == AWSRC_VARIANT_PF && KS >= 4) ? 1 : 2)
+__global__ void __launch_bounds__(32 * kMmaWarps, mma_per_sm(VAR, KS))
     search_mma_kernel(Prm pr, const __grid_constant__ LaunchDesc ld, const uint64_t* __restrict__ masks,
                       const float4* __restrict__ pairs, awsrc_candidate* __restrict__ cands, int64_t n_items,
                       int mode, MmaSlots sl, int tab_bytes) {
@@ -605,7 +608,7 @@ cudaError_t launch_mma_t(const Prm& pr, const LaunchDesc& ld, const uint64_t* ma
                          int64_t n_items, awsrc_candidate* cands, cudaStream_t st) {
   constexpr bool PF = VAR == AWSRC_VARIANT_PF;
   constexpr int V = KS == 1 ? 4 : 8, NV = 4 * KS / V;
-  constexpr int most = (PF && KS >= 4) ? 1 : 2;  // blocks per SM the registers allow
+  constexpr int most = mma_per_sm(VAR, KS);
   int mode = kLoadAsync, wb = 2, w0b = 2;
   for (int i = 0; i < ld.n; ++i) {
     const ModDesc& m = ld.m[i];
