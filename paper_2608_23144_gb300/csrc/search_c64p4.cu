@@ -667,10 +667,10 @@ cudaError_t launch_bfrag_c64p4(const Prm& pr, const uint64_t* masks, void* out, 
 }
 
 cudaError_t launch_merge_candidates(const awsrc_candidate* pc, int nsplit, int64_t T, int64_t t0, int64_t t1,
-                                   awsrc_candidate* out, cudaStream_t st) {
+                                   bool early, awsrc_candidate* out, cudaStream_t st) {
   if (t1 <= t0) return cudaSuccess;
-  const cudaError_t e = launch_pdl(merge_kernel, dim3((unsigned)((t1 - t0 + 255) / 256)), dim3(256), 0, st, pc, nsplit,
-                                   T, t0, t1, out);
+  const cudaError_t e = launch_dep(early, merge_kernel, dim3((unsigned)((t1 - t0 + 255) / 256)), dim3(256), 0, st, pc,
+                                   nsplit, T, t0, t1, out);
   note_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
