@@ -718,11 +718,20 @@ struct SelLayout {
   size_t bar, per_mod, bins, zero, seg, cnt, k0, v0, k1, v1, hist, total, bytes;
 };
 
+// Blocks worth launching: two rounds of tiles each (a barrier costs more, the more
+// blocks meet at it), but one per segment at least, since a segment's bins, offsets and
+// runs cost a block some microseconds however few tiles it has (700 modules of 7 tiles in
+// three blocks took 4270 us).
+int64_t want_blocks(const SelectPlan& sp, bool pf) {
+  const int64_t by_tiles = (sp.T + 4 * ST - 1) / (4 * ST), by_segments = pf ? 1 : std::min<int64_t>(sp.n_mod, sp.T);
+  return std::min(kMaxBlocks, std::max(by_tiles, by_segments));
+}
+
 SelLayout select_layout(const SelectPlan& sp, bool pf) {
   const size_t nseg = pf ? 1 : (size_t)sp.n_mod, T = (size_t)sp.T;
-  // one run per block, or kRunMin keys each, and a shorter one per segment
-  // (rows of kBins counters for step 1: one per block and segment it meets, fewer)
-  const size_t runs = std::min((size_t)kMaxBlocks, T / kRunMin) + 1 + nseg;
+  // sort runs: one per block, and a shorter one per segment; rows of kBins counters for
+  // step 1: row (block + segment) for each pair that meets, at most blocks + nseg - 1
+  const size_t runs = (size_t)want_blocks(sp, pf) + 1 + nseg;
   SelLayout l;
   size_t off = kStatusBytes;
   auto take = [&off](size_t n) {
@@ -816,10 +825,8 @@ awsrc_status select_run(const Prm& pr, const SelectPlan& sp, const int64_t* tile
       (e = cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, select_kernel, ST, smem);
   if (e != cudaSuccess) return cuda_fail(e, "select");
-  // as many blocks as are resident at once, fewer when a block would get less
-  // than two rounds of tiles (a barrier costs more, the more blocks meet at it)
-  const int64_t want = (sp.T + 4 * ST - 1) / (4 * ST);
-  const int64_t grid = std::max<int64_t>(1, std::min({want, (int64_t)stream_sms(st, nsm) * per_sm, kMaxBlocks}));
+  // at most as many blocks as are resident at once
+  const int64_t grid = std::max<int64_t>(1, std::min(want_blocks(sp, pf), (int64_t)stream_sms(st, nsm) * per_sm));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(ST);
