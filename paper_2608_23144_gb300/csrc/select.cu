@@ -89,6 +89,7 @@ struct GridBarrier {
   uint64_t limit_ns;
   __device__ bool sync() {
     __syncthreads();
+    if (gridDim.x == 1) return true;  // the only block has arrived
     bool ok = true;
     if (threadIdx.x == 0) {
       __threadfence();
