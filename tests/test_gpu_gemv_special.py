@@ -171,3 +171,20 @@ def test_bits_do_not_depend_on_the_batch(cols):
     both = aw.awsrc_packed_gemv_batch(prm, shapes, [(0, bbs[0], xs[0]), (1, bbs[1], xs[1])])
     for m in (0, 1):
         assert torch.equal(both[m], aw.awsrc_packed_gemv(prm, shapes, m, bbs[m], xs[m]))
+
+
+@pytest.mark.parametrize("C", [16, 32, 64])
+def test_smallest_record_scale(orc, C):
+    """Records at e = -126 alone (a zero backbone): the operand k_j 2^(e - S) is a
+    subnormal BF16, and the products with large inputs are in the ordinary range."""
+    import paper_2608_23144_gb300 as aw
+    rng = np.random.default_rng(85)
+    rows, cols, M = 40, 256, 8
+    W = np.zeros((rows, cols), np.float32)
+    gemv, definition = _setup(aw, orc, dict(C=C, P=4, b=4, S=64), W, rng.random(W.size // C) < 0.5, -126,
+                              lambda T: rng.integers(-7, 8, (T, 4)), rng)
+    x = (rng.uniform(0.5, 1, (M, cols)) * 2.0 ** 110).astype(np.float32)
+    y = gemv(x)
+    want, yabs = definition(x)
+    assert np.abs(want).max() > 2.0 ** -18
+    assert (np.abs(y - want) <= _bound(cols, C, yabs)).all()
