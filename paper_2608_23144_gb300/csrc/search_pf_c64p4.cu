@@ -335,7 +335,10 @@ __device__ __forceinline__ float pf_winner(const Prm& pr, const Smem& sm, int m,
   return odd ? g.y : g.x;
 }
 
-template <bool FAST>
+// STALL: the loader issues no copies from chunk pr.stall_chunk on (a test of the waits).
+// An instance of its own: with the comparison in the loader of every call, however it
+// is written, the search lost 3% (8.61 -> 8.85 ms on an attention block of a 7B layer).
+template <bool FAST, bool STALL>
 __global__ void __launch_bounds__(NT, 1)
     search_pf_kernel(Prm pr, LaunchDesc ld, const unsigned char* __restrict__ atoms,
                      const unsigned char* __restrict__ prods, const uint64_t* __restrict__ masks,
@@ -394,7 +397,7 @@ __global__ void __launch_bounds__(NT, 1)
     ++issued;
   };
   if (warp == EW + 1 && lane == 0)
-    while (issued < STAGES && issued < nck && issued != pr.stall_chunk) load_chunk();
+    while (issued < STAGES && issued < nck && !(STALL && issued == pr.stall_chunk)) load_chunk();
   // stage y = d * r and d, d = w_act * a + w_fisher * F (per element)
   for (int e = tid; e < BM * 64; e += NT) {
     const int r = e >> 6, j = e & 63;
@@ -504,7 +507,7 @@ __global__ void __launch_bounds__(NT, 1)
   } else if (warp == EW + 1) {
     // --------------------------------------------------------------- loader --
     if (lane == 0) {
-      while (issued < nck && issued != pr.stall_chunk) {  // the stage of chunk issued - STAGES, once its MMAs are complete
+      while (issued < nck && !(STALL && issued == pr.stall_chunk)) {  // the stage of chunk issued - STAGES, once its MMAs are complete
         if (!mbar_wait(&sm.sfree[issued % STAGES], (uint32_t)((issued / STAGES - 1) & 1), pr.wait_ns)) { timed_out = true; break; }
         load_chunk();
       }
@@ -699,7 +702,9 @@ cudaError_t launch_search_pf_c64p4(const Prm& pr, const LaunchDesc& ld, const vo
                                    const uint64_t* masks, int64_t n_blocks, awsrc_candidate* cands,
                                    uint32_t* status, cudaStream_t st) {
   const size_t smem = sizeof(Smem) + 1024;
-  auto kern = pr.fast_pow2 ? search_pf_kernel<true> : search_pf_kernel<false>;
+  auto kern = pr.stall_chunk >= 0 ? search_pf_kernel<false, true>
+              : pr.fast_pow2      ? search_pf_kernel<true, false>
+                                  : search_pf_kernel<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)n_blocks, NT, smem, st>>>(pr, ld, static_cast<const unsigned char*>(atoms),
