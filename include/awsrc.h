@@ -437,13 +437,19 @@ awsrc_status awsrc_decode_apply_inplace_noalloc(const awsrc_params* prm, int32_t
  *   faults are reported through awsrc_workspace_status(workspace).
  * awsrc_packed_gemv — y[m][i] = sum_j (W0_ij + r_ij) x[m][j] for module `m` of
  *   the list and the M <= 8 vectors x[m] (rows of x, M x cols, 16-byte
- *   aligned; y is M x rows): W0_ij = fl(q_ij * s_eff) from the packed backbone
- *   (awsrc_rtn_quantize's outputs; binary16 scales or SDQ), r_ij =
- *   fl(fl(k_j * C^-1/2) * scale) on the tiles the sidecar names (none when
- *   `sidecar` is NULL), both accumulated in binary32 (the residual terms in
- *   their own sums; x enters the sums unrounded). The result equals the double-precision product
- *   sum_j (W0_ij + r_ij) x_j, r_ij = k_j C^-1/2 scale, within
- *   (cols / min(C, 32) + 32) * 2^-24 * sum_j (|W0_ij x_j| + |r_ij x_j|).
+ *   aligned; y is M x rows): W0 from the packed backbone (awsrc_rtn_quantize's
+ *   outputs; binary16 scales or SDQ), r = k_j * C^-1/2 * scale on the tiles the
+ *   sidecar names (none when `sidecar` is NULL). Two kernels form it, chosen by
+ *   the parameters, M and the shapes of the module list (not by the tasks of a
+ *   call): the FP32 pipes, and for M >= 3 on lists with enough weights, P = 4,
+ *   b <= 5, C in {16, 32, 64} and power-of-two scales the tensor cores. Either
+ *   way x enters unrounded (the tensor cores take it as three BF16 parts, and
+ *   the FP32 pipes the inputs that three parts cannot hold), the codes' products
+ *   are summed in binary32 before a group's scale is applied, the residual has
+ *   its own sums, and the result equals the double-precision product
+ *   sum_j (W0_ij + r_ij) x_j, W0_ij = fl(q_ij * s_eff), within
+ *   (cols / min(C, 32) + 32) * 2^-24 * sum_j (|W0_ij x_j| + |r_ij x_j|)
+ *   while nothing overflows or leaves the normal range.
  *   The module needs cols % 128 == 0.
  * Errors: INVALID_ARG, SHAPE, UNSUPPORTED, WORKSPACE, CUDA.
  */
@@ -467,12 +473,12 @@ awsrc_status awsrc_packed_gemv(const awsrc_params* prm, int32_t n_mod, const aws
 
 /*
  * awsrc_packed_gemv_batch — awsrc_packed_gemv for 1 <= n_task <= 16 tasks in
- * one launch (tasks whose M x cols inputs exceed 96 KB take one more launch
- * each): task i computes y_i = (W0 + r_hat) x_i for module tasks[i].m with
+ * one launch (on the FP32 pipes, tasks whose M x cols inputs exceed 96 KB take
+ * one more launch each): task i computes y_i = (W0 + r_hat) x_i for module tasks[i].m with
  * its packed backbone tasks[i].pw, all with the same sidecar and M. Tasks may
  * name the same module and share x (the q/k/v or gate/up projections of one
  * input); y arrays must not overlap each other or any input. Each y_i is
- * bit-identical to the single call's. Errors: as awsrc_packed_gemv;
+ * bit-identical to the single call's on the same module list. Errors: as awsrc_packed_gemv;
  * UNSUPPORTED for n_task > 16.
  */
 typedef struct awsrc_gemv_task {

@@ -131,7 +131,8 @@ EncodeLayout encode_layout(const Prm& pr, int32_t n_mod, const awsrc_module* mod
                        : L.spec_pf ? pr.S_pad / search_pf_c64p4_chunk()
                        : L.mma     ? (pr.S + 7) / 8  // groups of eight seeds
                                    : (pr.S + gs.lanes - 1) / gs.lanes;
-  int64_t ns = L.mma ? mma_splits(base_blocks, units, search_mma_slots(pr)) : (kTargetBlocks + base_blocks - 1) / base_blocks;
+  int64_t ns = (kTargetBlocks + base_blocks - 1) / base_blocks;
+  if (L.mma) ns = mma_splits(base_blocks, units, search_mma_slots(pr));
   ns = std::max<int64_t>(1, std::min<int64_t>(ns, units));
   L.nsplit = (int)ns;
   size_t off = kStatusBytes;

@@ -114,11 +114,12 @@ __host__ __device__ constexpr int gram_stride(int P) {
   return ((P * (P - 1) + P + 1) + 3) / 4 * 4;
 }
 
-// float2 entries per (column block, seed pair) of the paired table the C = 64,
-// P = 4 search streams: -L, invD rounded up after multiplying by the seed's
-// pruning-bound multiplier (used only by the bound), invD, G off-diagonal
-// (2*G_pq on the fast power-of-two path), gd, zero padding to an even count;
-// seed 2i in component x and seed 2i+1 in y.
+// float2 entries per (column block, seed pair) of the paired table that the C = 64,
+// P = 4 U search streams and the mma.sync U searches read: -L, invD rounded up
+// after multiplying by the seed's pruning-bound multiplier (used only by the bound,
+// which the mma.sync searches do not have), invD, G off-diagonal (2*G_pq on the
+// fast power-of-two path), gd, zero padding to an even count; seed 2i in component x
+// and seed 2i+1 in y.
 __host__ __device__ constexpr int pair_stride(int P) {
   return ((P * (P - 1) + 2 * P + 1) + 1) / 2 * 2;
 }

@@ -579,7 +579,8 @@ cudaError_t launch_gram_p(const Prm& pr, const LaunchDesc& ld, const uint64_t* m
   // early while the tables are small (1.3 us less at 256 seeds and two column blocks);
   // from 1024 seeds on, blocks placed while the kernels before still run come to share
   // SMs (64 x 128, S = 1024: 31 -> 35 us, 1024 x 1024: 177 -> 181)
-  const cudaError_t e = launch_dep(pr.S_pad < 1024, gram_u_kernel<P>, grid, dim3(128), 0, st, pr, ld, masks, gram, pairs);
+  const cudaError_t e = launch_dep(pr.S_pad < 1024, gram_u_kernel<P>, grid, dim3(128), 0, st, pr, ld, masks, gram,
+                                   pairs);
   note_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

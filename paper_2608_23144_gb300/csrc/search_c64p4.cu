@@ -690,8 +690,8 @@ cudaError_t launch_search_c64p4(const Prm& pr, const LaunchDesc& ld, const void*
   // early while the call fits one wave, where launches count (a 256 x 512 matrix with
   // 256 seeds: 41 -> 31 us with the whole chain early); with more tile blocks the CTAs
   // that start during the table kernels only disturb them (8661 -> 8686 us a 3B layer)
-  e = launch_dep(n_blocks <= nsm, kern, dim3((unsigned)grid), dim3(NT), smem, st, pr, ld, n_blocks, static_cast<const uint4*>(table),
-                 pairs, masks, cands, status);
+  e = launch_dep(n_blocks <= nsm, kern, dim3((unsigned)grid), dim3(NT), smem, st, pr, ld, n_blocks,
+                 static_cast<const uint4*>(table), pairs, masks, cands, status);
   note_launches(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

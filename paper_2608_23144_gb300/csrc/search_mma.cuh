@@ -549,7 +549,8 @@ __global__ void __launch_bounds__(32 * kMmaWarps, mma_per_sm(VAR, KS))
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
             ldl_solve2<P>(nL[r], invD[r], bv[r], alpha[r]);
-            gp[r] = mma_gain<P, FAST, false>(pr, alpha[r], bv[r], make_float2(row[r].gd, row[r].gd), G[r], cw[r], sf[r]);
+            gp[r] = mma_gain<P, FAST, false>(pr, alpha[r], bv[r], make_float2(row[r].gd, row[r].gd), G[r], cw[r],
+                                             sf[r]);
             if (!okx[r]) gp[r].x = ninf();
             if (!oky[r]) gp[r].y = ninf();
           }
@@ -573,8 +574,18 @@ __global__ void __launch_bounds__(32 * kMmaWarps, mma_per_sm(VAR, KS))
         // seeds reach a thread in increasing order: a strictly greater gain wins
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
-          if (s < pr.S && gp[r].x > bg[r]) { bg[r] = gp[r].x; bs[r] = (uint32_t)s; bc[r] = cw[r][0]; bf[r] = sf[r][0]; }
-          if (s + 1 < pr.S && gp[r].y > bg[r]) { bg[r] = gp[r].y; bs[r] = (uint32_t)s + 1; bc[r] = cw[r][1]; bf[r] = sf[r][1]; }
+          if (s < pr.S && gp[r].x > bg[r]) {
+            bg[r] = gp[r].x;
+            bs[r] = (uint32_t)s;
+            bc[r] = cw[r][0];
+            bf[r] = sf[r][0];
+          }
+          if (s + 1 < pr.S && gp[r].y > bg[r]) {
+            bg[r] = gp[r].y;
+            bs[r] = (uint32_t)s + 1;
+            bc[r] = cw[r][1];
+            bf[r] = sf[r][1];
+          }
         }
       }
     }

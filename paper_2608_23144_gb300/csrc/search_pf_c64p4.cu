@@ -488,7 +488,10 @@ __global__ void __launch_bounds__(NT, 1)
     for (; k < nck; ++k) {
       const int st = k % STAGES, tb = k & 1;
       if (!mbar_wait_warp(&sm.full[st], (uint32_t)((k / STAGES) & 1), pr.wait_ns)) { timed_out = true; break; }
-      if (k >= 2 && !mbar_wait_warp(&sm.tempty[tb], (uint32_t)(((k - 2) >> 1) & 1), pr.wait_ns)) { timed_out = true; break; }
+      if (k >= 2 && !mbar_wait_warp(&sm.tempty[tb], (uint32_t)(((k - 2) >> 1) & 1), pr.wait_ns)) {
+        timed_out = true;
+        break;
+      }
       tc_fence_after();
       const uint32_t sa = smem_addr(&sm.stage[st][0]), sq = sa + kABytes;
       const uint32_t acc = tm + (uint32_t)(tb * 256);
@@ -507,8 +510,12 @@ __global__ void __launch_bounds__(NT, 1)
   } else if (warp == EW + 1) {
     // --------------------------------------------------------------- loader --
     if (lane == 0) {
-      while (issued < nck && !(STALL && issued == pr.stall_chunk)) {  // the stage of chunk issued - STAGES, once its MMAs are complete
-        if (!mbar_wait(&sm.sfree[issued % STAGES], (uint32_t)((issued / STAGES - 1) & 1), pr.wait_ns)) { timed_out = true; break; }
+      // each time the stage of chunk issued - STAGES, once its MMAs are complete
+      while (issued < nck && !(STALL && issued == pr.stall_chunk)) {
+        if (!mbar_wait(&sm.sfree[issued % STAGES], (uint32_t)((issued / STAGES - 1) & 1), pr.wait_ns)) {
+          timed_out = true;
+          break;
+        }
         load_chunk();
       }
       // the copies in flight land before the block ends, whoever timed out
