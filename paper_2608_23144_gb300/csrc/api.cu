@@ -106,9 +106,11 @@ int64_t mma_splits(int64_t base, int64_t units, int64_t slots) {
     return tenths * ((units + ns - 1) / ns + 4) + 2 * ns;
   };
   int64_t best = most;
-  for (int64_t ns = 1; ns < most; ++ns) {
-    const int64_t per = (units + ns - 1) / ns;
-    if ((units + per - 1) / per == ns && cost(ns) < cost(best)) best = ns;  // (no empty splits)
+  for (int64_t ns = 1; ns < most;) {  // each number of groups an item can have, with its fewest splits
+    if (cost(ns) < cost(best)) best = ns;
+    const int64_t per = (units + ns - 1) / ns - 1;
+    if (per < 1) break;
+    ns = (units + per - 1) / per;
   }
   return 10 * cost(best) <= 9 * cost(most) ? best : most;
 }
