@@ -93,13 +93,20 @@ struct EncodeLayout {
 // one or two groups of seeds and the merge a hundred candidates of every tile (1024
 // tiles of 16, S = 1024, P = 2: 56 us in 128 splits, 26 in 38), where too few leave a
 // wave nearly empty (8192 tiles, S = 4096: 150 us in 19 splits, 198 in 5). So calls of at
-// most one run per slot take the least of, in groups, waves x (an item's groups + 4) + a
-// fifth per split, if that is 10% less; a last wave that is filled to less than a third
-// counts as 0.6. (Not where an SM holds one block, P_F with C = 64 and 128: its groups
-// are dear, and fewer splits cost up to 20%.)
+// most half a run per slot take the least of, in groups, waves x (an item's groups + 4) +
+// a fifth per split, if that is 20% less; a last wave that is filled to less than a
+// third counts as 0.6. Where an SM holds one block (P_F with C = 64 and 128) a group is dearer
+// against the rest: calls of at most a quarter of a run per slot take the fewest whole
+// waves that splits fill to 93% (64 x 256, C = 64, P = 2, S = 4096: 152 us in 256 splits,
+// 112 on the scalar search, 32 in 76).
 int64_t mma_splits(int64_t base, int64_t units, int64_t slots) {
   const int64_t most = std::max<int64_t>(1, std::min((kTargetBlocks + base - 1) / base, units));
-  if (base > slots || slots <= kSms) return most;
+  if (slots <= kSms) {
+    for (int64_t w = 1; 4 * base <= slots && w * slots <= kTargetBlocks; ++w)
+      if (100 * (w * slots / base) * base >= 93 * w * slots) return std::min(w * slots / base, units);
+    return most;
+  }
+  if (2 * base > slots) return most;
   auto cost = [&](int64_t ns) {
     const int64_t items = ns * base, full = items / slots, rest = items % slots;
     const int64_t tenths = 10 * full + (rest == 0 ? 0 : full > 0 && 10 * rest <= 3 * slots ? 6 : 10);
@@ -112,7 +119,7 @@ int64_t mma_splits(int64_t base, int64_t units, int64_t slots) {
     if (per < 1) break;
     ns = (units + per - 1) / per;
   }
-  return 10 * cost(best) <= 9 * cost(most) ? best : most;
+  return 10 * cost(best) <= 8 * cost(most) ? best : most;
 }
 
 EncodeLayout encode_layout(const Prm& pr, int32_t n_mod, const awsrc_module* mods, int64_t T) {

@@ -11,7 +11,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("C,P,S,shape,variant", [
     (16, 2, 1024, (9, 64), 0), (16, 4, 777, (64, 64), 0), (16, 4, 2051, (16, 128), 1), (32, 2, 300, (130, 128), 1),
-    (32, 4, 4096, (3, 64), 0), (64, 2, 1000, (20, 64), 0), (64, 2, 600, (40, 128), 1), (128, 4, 500, (10, 256), 1),
+    (32, 4, 4096, (3, 64), 0), (64, 2, 1000, (20, 64), 0), (64, 2, 600, (40, 128), 1), (64, 2, 4000, (16, 64), 1),
+    (128, 4, 1500, (10, 256), 1),
 ])
 def test_candidates_match_oracle(orc, C, P, S, shape, variant):
     import paper_2608_23144_gb300 as aw
