@@ -32,10 +32,11 @@
 // else is in the launch, the product's bits do not.
 //
 // One 3B-shaped layer (77 M weights, 0.162 bits/weight of records, SDQ scales, eight
-// vectors, one batched launch): 308 -> 79 us a call. Its
-// relative error against 64 bits is 9.6e-8 where the FP32 pipes' sums had 1.4e-7.
-// Bound by issue (46% of slots): 370 instructions per 16 rows and 128 inputs for the
-// backbone (half of them the split of x) and up to 380 for the residual.
+// vectors, one batched launch): 308 -> 76 us a call. Its relative error against 64 bits
+// is 9.7e-8 where the FP32 pipes' sums had 1.4e-7. Bound by latency and issue (43% of
+// slots): 695 warp instructions per 16 rows and 128 inputs without records (the split of
+// x about half), 910 on average with this layer's; x comes from L1, so the sums' shared
+// memory is no larger than needed (32 KB a block for all cases: 3 to 6% slower).
 #include <algorithm>
 
 #include "codetab.cuh"
@@ -208,7 +209,8 @@ __device__ __forceinline__ void run_fp32(const float* x, int64_t cols, unsigned 
 
 template <int LC>
 __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const __grid_constant__ GemvArgs a, int M) {
-  __shared__ float4 part[kWarps][kSums][32];  // [row tile of the block][sum][lane]
+  extern __shared__ float4 part_mem[];
+  float4(*part)[kSums][32] = reinterpret_cast<float4(*)[kSums][32]>(part_mem);  // [row tile of the block][sum][lane]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
   int ti = 0;
   for (int i = 1; i < a.n_task; ++i)
@@ -219,10 +221,8 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
   const int gpr = (int)(tk.cols >> 7);
   // the warp's groups: kSums / ks of the row tile's eight sums (some empty when gpr < 8)
   auto bound = [gpr](int i) { return (int)((int64_t)gpr * i / kSums); };
-  int sum = kSums / ks * slice;
-  const int g0 = bound(sum), g1 = row0 < tk.rows ? bound(sum + kSums / ks) : g0;
-  while (sum < kSums - 1 && bound(sum + 1) <= g0) ++sum;  // the sum that holds group g0
-  int sum_end = bound(sum + 1);
+  const int sum0 = kSums / ks * slice, sum1 = row0 < tk.rows ? sum0 + kSums / ks : sum0;
+  const int g0 = bound(sum0), g1 = bound(sum1);
   int64_t row[2];
 #pragma unroll
   for (int r = 0; r < 2; ++r) row[r] = min(row0 + g + 8 * r, tk.rows - 1);  // rows past the end repeat the last one
@@ -261,115 +261,114 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
   };
   // c = 2^-(LC/2) is folded into the residual for C = 64 and 16; C = 32 had 1/8
   const float cf = LC == 5 ? __fmul_rn(8.0f, pr.c) : 1.0f;
-  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, racc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   if (g0 < g1) load(g0);
-  for (int gr = g0; gr < g1; ++gr) {
-    uint32_t wc[2][4];
-    unsigned long long ec[2][NT];
-    const float sc[2] = {s[0], s[1]};
+  int gr = g0;
+  for (int sum = sum0; sum < sum1; ++sum) {
+    const int end = bound(sum + 1);
+    if (gr == end) continue;
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, racc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    for (; gr < end; ++gr) {
+      uint32_t wc[2][4];
+      unsigned long long ec[2][NT];
+      const float sc[2] = {s[0], s[1]};
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
+      for (int r = 0; r < 2; ++r) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) wc[r][j] = w[r][j];
+        for (int j = 0; j < 4; ++j) wc[r][j] = w[r][j];
 #pragma unroll
-      for (int t = 0; t < NT; ++t) ec[r][t] = e[r][t];
-    }
-    if (gr + 1 < g1) load(gr + 1);
-    float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    float rh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    TileRec tr[2];
-    XRange xr{0.0f, 0u};
-    bool any = false;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      float4 xa = make_float4(0.0f, 0.0f, 0.0f, 0.0f), xb = xa;
-      if (live) {
-        xa = __ldg(reinterpret_cast<const float4*>(xp + 128 * gr + 32 * j));
-        xb = __ldg(reinterpret_cast<const float4*>(xp + 128 * gr + 32 * j + 4));
+        for (int t = 0; t < NT; ++t) ec[r][t] = e[r][t];
       }
-      const int t = LC == 6 ? j >> 1 : j;
-      if (LC != 6 || (j & 1) == 0) {  // a new tile
-        any = mp[0] && __any_sync(0xffffffffu, (ec[0][t] | ec[1][t]) != 0ull);
-        if (any) {
-          tr[0] = tile_rec<LC>(a, ec[0][t]);
-          tr[1] = tile_rec<LC>(a, ec[1][t]);
-        }
-      }
-      uint4 nb[2];
-      if (any) {
-        const int win = ((32 * j + 8 * q) & ((1 << LC) - 1)) >> 3;
+      if (gr + 1 < g1) load(gr + 1);
+      float h[4] = {0.0f, 0.0f, 0.0f, 0.0f}, ml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      float rh[4] = {0.0f, 0.0f, 0.0f, 0.0f}, rml[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+      TileRec tr[2];
+      XRange xr{0.0f, 0u};
+      bool any = false;
 #pragma unroll
-        for (int r = 0; r < 2; ++r) nb[r] = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + win);
-      }
-      BRun b;
-      split_run(xa, xb, b, xr);
-      uint32_t c0[4], c1[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        c0[i] = code_pair(wc[0][j], i);
-        c1[i] = code_pair(wc[1][j], i);
-      }
-      mma_run(h, ml, c0, c1, b);
-      if (any) {
-        residual_pairs(tr[0], nb[0], c0);
-        residual_pairs(tr[1], nb[1], c1);
-        mma_run(rh, rml, c0, c1, b);
-      }
-    }
-    // Vectors that the MMAs could not take (inputs too small for the split, too large for
-    // the sums, an infinity or NaN) get the group again on the FP32 pipes. Their columns
-    // of the accumulators are their own.
-    const unsigned odd = __ballot_sync(0xffffffffu, !xr.ok());
-    if (odd) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if ((odd >> (8 * q + 4 * (i & 1))) & 15u) h[i] = ml[i] = rh[i] = rml[i] = 0.0f;
-#pragma unroll 1
       for (int j = 0; j < 4; ++j) {
-        const float* xj = tk.x + 128 * gr + 32 * j + 8 * q;
+        float4 xa = make_float4(0.0f, 0.0f, 0.0f, 0.0f), xb = xa;
+        if (live) {
+          xa = __ldg(reinterpret_cast<const float4*>(xp + 128 * gr + 32 * j));
+          xb = __ldg(reinterpret_cast<const float4*>(xp + 128 * gr + 32 * j + 4));
+        }
+        const int t = LC == 6 ? j >> 1 : j;
+        if (LC != 6 || (j & 1) == 0) {  // a new tile
+          any = mp[0] && __any_sync(0xffffffffu, (ec[0][t] | ec[1][t]) != 0ull);
+          if (any) {
+            tr[0] = tile_rec<LC>(a, ec[0][t]);
+            tr[1] = tile_rec<LC>(a, ec[1][t]);
+          }
+        }
+        uint4 nb[2];
+        if (any) {
+          const int win = ((32 * j + 8 * q) & ((1 << LC) - 1)) >> 3;
+#pragma unroll
+          for (int r = 0; r < 2; ++r) nb[r] = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + win);
+        }
+        BRun b;
+        split_run(xa, xb, b, xr);
         uint32_t c0[4], c1[4];
-        float o[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          c0[i] = code_pair(__ldg(cp[0] + 16 * gr + 4 * j), i);
-          c1[i] = code_pair(__ldg(cp[1] + 16 * gr + 4 * j), i);
+          c0[i] = code_pair(wc[0][j], i);
+          c1[i] = code_pair(wc[1][j], i);
         }
-        run_fp32(xj, tk.cols, odd, q, c0, c1, true, true, o);
+        mma_run(h, ml, c0, c1, b);
+        if (any) {
+          residual_pairs(tr[0], nb[0], c0);
+          residual_pairs(tr[1], nb[1], c1);
+          mma_run(rh, rml, c0, c1, b);
+        }
+      }
+      // Vectors that the MMAs could not take (inputs too small for the split, too large for
+      // the sums, an infinity or NaN) get the group again on the FP32 pipes. Their columns
+      // of the accumulators are their own.
+      const unsigned odd = __ballot_sync(0xffffffffu, !xr.ok());
+      if (odd) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (sc[i >> 1] != 0.0f) acc[i] = __fmaf_rn(o[i], sc[i >> 1], acc[i]);
-        if (!mp[0]) continue;
-        unsigned long long en[2];
-        const int jt = 32 * j + 8 * q;  // the thread's first input in the group
+          if ((odd >> (8 * q + 4 * (i & 1))) & 15u) h[i] = ml[i] = rh[i] = rml[i] = 0.0f;
+#pragma unroll 1
+        for (int j = 0; j < 4; ++j) {
+          const float* xj = tk.x + 128 * gr + 32 * j + 8 * q;
+          uint32_t c0[4], c1[4];
+          float o[4];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          en[r] = __ldg(mp[r] + ((128 * gr + jt) >> LC));
-          tr[r] = tile_rec<LC>(a, en[r]);
-          const uint4 nb = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + ((jt & ((1 << LC) - 1)) >> 3));
-          residual_pairs(tr[r], nb, r ? c1 : c0);
+          for (int i = 0; i < 4; ++i) {
+            c0[i] = code_pair(__ldg(cp[0] + 16 * gr + 4 * j), i);
+            c1[i] = code_pair(__ldg(cp[1] + 16 * gr + 4 * j), i);
+          }
+          run_fp32(xj, tk.cols, odd, q, c0, c1, true, true, o);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (sc[i >> 1] != 0.0f) acc[i] = __fmaf_rn(o[i], sc[i >> 1], acc[i]);
+          if (!mp[0]) continue;
+          unsigned long long en[2];
+          const int jt = 32 * j + 8 * q;  // the thread's first input in the group
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            en[r] = __ldg(mp[r] + ((128 * gr + jt) >> LC));
+            tr[r] = tile_rec<LC>(a, en[r]);
+            const uint4 nb = __ldg(a.nib + ((size_t)tr[r].seed << (LC - 3)) + ((jt & ((1 << LC) - 1)) >> 3));
+            residual_pairs(tr[r], nb, r ? c1 : c0);
+          }
+          run_fp32(xj, tk.cols, odd, q, c0, c1, en[0] != 0ull, en[1] != 0ull, o);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) racc[i] = __fadd_rn(racc[i], o[i]);
         }
-        run_fp32(xj, tk.cols, odd, q, c0, c1, en[0] != 0ull, en[1] != 0ull, o);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) racc[i] = __fadd_rn(racc[i], o[i]);
       }
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      // an all-zero group (scale 0) adds nothing, whatever x holds
-      const float sr = sc[i >> 1];
-      if (sr != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sr, acc[i]);
-      racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
-    }
-    if (gr + 1 == sum_end) {
-      float v[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        v[i] = __fmaf_rn(racc[i], cf, acc[i]);
-        acc[i] = racc[i] = 0.0f;
+        // an all-zero group (scale 0) adds nothing, whatever x holds
+        const float sr = sc[i >> 1];
+        if (sr != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sr, acc[i]);
+        racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
       }
-      part[warp / ks][sum][lane] = make_float4(v[0], v[1], v[2], v[3]);
-      while (sum < kSums - 1 && sum_end <= gr + 1) sum_end = bound(++sum + 1);
     }
+    float v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __fmaf_rn(racc[i], cf, acc[i]);
+    part[warp / ks][sum][lane] = make_float4(v[0], v[1], v[2], v[3]);
   }
   __syncthreads();
   float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
@@ -405,9 +404,9 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
 //  * on the FP32 pipes 3 + (0.3 + 0.21 M) per million weights, and M where the inputs do
 //    not fit in shared memory (gemv.cu).
 // Measured, FP32 pipes against tensor cores: 1024 x 1024, M = 4: 4.6 and 6.3; 2048 x
-// 2048, M = 3 and 8: 8.0 and 9.9, 14.2 and 10.2; 512 x 11008, M = 4 and 8: 20.3 and 37.7,
-// 38.4 and 38.8; 11008 x 2048, M = 3 and 5: 24.4 and 28.7, 33.0 and 29.2; the layer above,
-// M = 3 and 8: 125 and 77, 267 and 78.
+// 2048, M = 3 and 8: 8.0 and 9.9, 14.2 and 9.9; 512 x 11008, M = 4 and 8: 20.1 and 36,
+// 38.4 and 36; 11008 x 2048, M = 3 and 5: 24.3 and 26.5, 32.9 and 26.8; the layer above
+// (random records), M = 3 and 8: 126 and 73, 268 and 76.
 bool gemv_mma(const Prm& pr, const GemvArgs& a, int M, int n_mod, const awsrc_module* mods) {
   const bool c = pr.C == 16 || pr.C == 32 || pr.C == 64;
   if (M < 3 || !c || (a.map && (!a.nib || pr.scale_mode != AWSRC_SCALE_POW2))) return false;
@@ -427,46 +426,73 @@ cudaError_t launch_gemv_mma(const Prm& pr, const GemvArgs& a, int M, cudaStream_
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  // Slices of at most eight groups (of four: 84 us instead of 77 on the layer above), and
-  // shorter ones while the launch has less than 1.75 waves of warps: a warp takes 2 to
-  // 3.4 us per group however empty the chip is, so a 2048 x 2048 module alone went from
-  // 29 us (two slices) to 10 (eight), an 11008 x 2048 one from 35 to 29, a gate and up pair
-  // (now four slices) from 59 to 52.
-  int64_t warps = 0;
-  auto tiles = [](const GemvTask& t) { return (t.rows + 15) / 16; };
-  auto groups = [](const GemvTask& t) { return ((t.cols >> 7) + t.slices - 1) / t.slices; };  // of a slice
-  for (int i = 0; i < b.n_task; ++i) {
-    GemvTask& t = b.t[i];
-    t.slices = 1;
-    while (t.slices < kWarps && groups(t) > 8) t.slices <<= 1;
-    warps += tiles(t) * t.slices;
-  }
-  while (warps < (int64_t)nsm * 2 * kWarps * 7 / 4) {
-    GemvTask* m = nullptr;  // the task with the longest slices
+  // Slices of at most eight groups; then the longest are halved, one task after the
+  // other, and the division of least estimated time is kept. A block takes, in us, 1.2
+  // and per group of its slices 3.3 alone on an SM, 4.4 beside another block, however
+  // empty the chip is: up to three blocks per SM go in whole rounds, more keep the SMs
+  // busy but for a quarter of a round. A 2048 x 2048 module alone went from 29 us (two
+  // slices) to 10 (eight), an 11008 x 2048 one from 35 to 27, q/k/v of a 3B layer from 28
+  // to 13; but a 3584-wide attention block takes 34 us in four slices (0.84 of the
+  // blocks that are resident at once) and 37 in eight.
+  int64_t tiles[kMaxGemvTasks] = {}, gpr[kMaxGemvTasks] = {};
+  int ls[kMaxGemvTasks] = {}, best[kMaxGemvTasks] = {};  // log2 of the slices
+  auto groups = [&](int i) { return (gpr[i] + (1 << ls[i]) - 1) >> ls[i]; };  // of a slice
+  auto estimate = [&]() {
+    double n = 0.0, work = 0.0, longest = 0.0;
     for (int i = 0; i < b.n_task; ++i) {
-      GemvTask& t = b.t[i];
-      if (t.slices < kWarps && groups(t) > 1 && (!m || groups(t) > groups(*m))) m = &t;
+      const double blk = (double)(((tiles[i] << ls[i]) + kWarps - 1) / kWarps), g = (double)groups(i);
+      n += blk;
+      work += blk * g;
+      longest = std::max(longest, g);
     }
-    if (!m) break;
-    warps += tiles(*m) * m->slices;
-    m->slices <<= 1;
+    const double pair = 4.4 * work / n + 1.2, one = 3.3 * work / n + 1.2;
+    const double t = n > 3.0 * nsm   ? (0.5 * n / nsm + 0.25) * pair
+                     : n > 2.0 * nsm ? pair + one
+                     : n > nsm       ? pair
+                                     : one;
+    return std::max(t, 3.3 * longest + 1.2);
+  };
+  for (int i = 0; i < b.n_task; ++i) {
+    tiles[i] = (b.t[i].rows + 15) / 16;
+    gpr[i] = b.t[i].cols >> 7;
+    ls[i] = 0;
+    while ((1 << ls[i]) < kWarps && groups(i) > 8) ++ls[i];
+    best[i] = ls[i];
   }
+  double least = estimate();
+  while (true) {
+    int m = -1;  // the task with the longest slices
+    for (int i = 0; i < b.n_task; ++i)
+      if ((1 << ls[i]) < kWarps && groups(i) > 1 && (m < 0 || groups(i) > groups(m))) m = i;
+    if (m < 0) break;
+    ++ls[m];
+    const double t = estimate();
+    if (t < 0.97 * least) {
+      least = t;
+      std::copy(ls, ls + b.n_task, best);
+    }
+  }
+  for (int i = 0; i < b.n_task; ++i) b.t[i].slices = 1 << best[i];
   // the tasks with the longest slices first, so that their blocks do not end the
   // launch (69 us in the caller's order, the down projection last)
-  std::stable_sort(b.t, b.t + b.n_task, [&](const GemvTask& x, const GemvTask& y) { return groups(x) > groups(y); });
+  std::stable_sort(b.t, b.t + b.n_task, [](const GemvTask& x, const GemvTask& y) {
+    return (x.cols >> 7) * y.slices > (y.cols >> 7) * x.slices;
+  });
   int64_t blocks = 0;
+  size_t smem = 0;  // as little as the slices need: the rest of the SM's memory caches x
   for (int i = 0; i < b.n_task; ++i) {
     GemvTask& t = b.t[i];
     const int64_t per = 16 * (kWarps / t.slices);
     t.block0 = (int)blocks;
+    smem = std::max(smem, (size_t)(kWarps / t.slices) * kSums * 32 * sizeof(float4));
     blocks += (t.rows + per - 1) / per;
   }
   if (blocks > 0x7fffffffll) return cudaErrorInvalidConfiguration;
   const dim3 grid((unsigned)blocks), block(32 * kWarps);
   switch (pr.C) {
-    case 16: gemv_mma_kernel<4><<<grid, block, 0, st>>>(pr, b, M); break;
-    case 32: gemv_mma_kernel<5><<<grid, block, 0, st>>>(pr, b, M); break;
-    case 64: gemv_mma_kernel<6><<<grid, block, 0, st>>>(pr, b, M); break;
+    case 16: gemv_mma_kernel<4><<<grid, block, smem, st>>>(pr, b, M); break;
+    case 32: gemv_mma_kernel<5><<<grid, block, smem, st>>>(pr, b, M); break;
+    case 64: gemv_mma_kernel<6><<<grid, block, smem, st>>>(pr, b, M); break;
     default: return cudaErrorInvalidValue;
   }
   note_launches(1);
