@@ -440,10 +440,8 @@ awsrc_status awsrc_decode_apply_inplace_noalloc(const awsrc_params* prm, int32_t
  *   aligned; y is M x rows): W0 from the packed backbone (awsrc_rtn_quantize's
  *   outputs; binary16 scales or SDQ), r = k_j * C^-1/2 * scale on the tiles the
  *   sidecar names (none when `sidecar` is NULL). Two kernels form it, chosen by
- *   the parameters, M and the shapes of the module list (not by the tasks of a
- *   call): the FP32 pipes, and for M >= 3 on lists with enough weights, P = 4,
- *   b <= 5, C in {16, 32, 64} and power-of-two scales the tensor cores. Either
- *   way x enters unrounded (the tensor cores take it as three BF16 parts, and
+ *   the parameters and M: the FP32 pipes, and for M >= 3, P = 4, b <= 5, C in
+ *   {16, 32, 64} and power-of-two scales the tensor cores. Either way x enters unrounded (the tensor cores take it as three BF16 parts, and
  *   the FP32 pipes the inputs that three parts cannot hold), the codes' products
  *   are summed in binary32 before a group's scale is applied, the residual has
  *   its own sums, and the result equals the double-precision product
@@ -478,7 +476,7 @@ awsrc_status awsrc_packed_gemv(const awsrc_params* prm, int32_t n_mod, const aws
  * its packed backbone tasks[i].pw, all with the same sidecar and M. Tasks may
  * name the same module and share x (the q/k/v or gate/up projections of one
  * input); y arrays must not overlap each other or any input. Each y_i is
- * bit-identical to the single call's on the same module list. Errors: as awsrc_packed_gemv;
+ * bit-identical to the single call's. Errors: as awsrc_packed_gemv;
  * UNSUPPORTED for n_task > 16.
  */
 typedef struct awsrc_gemv_task {

@@ -772,8 +772,8 @@ awsrc_status awsrc_packed_gemv_batch(const awsrc_params* prm, int32_t n_mod, con
     if ((s = gemv_task(pr, n_mod, mods, tasks[i].m, &tasks[i].pw, tasks[i].x, tasks[i].y, &a.t[i])) != AWSRC_OK)
       return s;
   if ((s = gemv_sidecar(prm, pr, n_mod, mods, T, sidecar, sidecar_bytes, &a)) != AWSRC_OK) return s;
-  const cudaError_t e = gemv_mma(pr, a, M, n_mod, mods) ? launch_gemv_mma(pr, a, M, (cudaStream_t)stream)
-                                                       : launch_gemv(pr, a, M, (cudaStream_t)stream);
+  const cudaError_t e = gemv_mma(pr, a, M) ? launch_gemv_mma(pr, a, M, (cudaStream_t)stream)
+                                          : launch_gemv(pr, a, M, (cudaStream_t)stream);
   return e == cudaSuccess ? AWSRC_OK : cuda_fail(e, "packed_gemv");
 }
 

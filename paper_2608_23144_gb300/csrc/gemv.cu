@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(32 * kGemvWarps, M <= 2 ? 3 : 1) gemv_warp_ker
 // Relative cost of a task: its weights.
 double task_cost(const GemvTask& t) { return (double)t.rows * (double)t.cols; }
 
-size_t x_smem_bytes(int64_t cols, int M) { return (size_t)M * ((cols + 1023) / 1024 * 1024) * 4; }
+size_t x_smem_bytes(const GemvTask& t, int M) { return (size_t)M * ((t.cols + 1023) / 1024 * 1024) * 4; }
 
 template <int M>
 cudaError_t launch_gemv_m(const Prm& pr, const GemvArgs& a, cudaStream_t st) {
@@ -467,8 +467,8 @@ cudaError_t launch_gemv_m(const Prm& pr, const GemvArgs& a, cudaStream_t st) {
   size_t smem = 0;
   double work = 0.0;
   for (int i = 0; i < a.n_task; ++i) {
-    const size_t need = x_smem_bytes(a.t[i].cols, M);
-    if (gemv_in_smem(a.t[i].cols, M)) {
+    const size_t need = x_smem_bytes(a.t[i], M);
+    if (need <= kGemvSmemMax) {
       b.t[b.n_task++] = a.t[i];
       smem = need > smem ? need : smem;
       work += task_cost(a.t[i]);
@@ -536,8 +536,6 @@ cudaError_t launch_gemv(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st
     default: return cudaErrorInvalidValue;
   }
 }
-
-bool gemv_in_smem(int64_t cols, int M) { return x_smem_bytes(cols, M) <= kGemvSmemMax; }
 
 bool gemv_tables(const Prm& pr) { return code_tables(pr) && pr.C >= 16; }
 

@@ -27,13 +27,13 @@
 // nibble-table window, two float4 of vector g.
 //
 // A warp takes 16 rows and a slice of the columns. A row tile's product is always made
-// of the same eight column sums, added in order through the shared memory of the block
+// of the same eight column sums, added two by two through the shared memory of the block
 // that has all its slices: how many slices there are (one to eight) depends on what
 // else is in the launch, the product's bits do not.
 //
 // One 3B-shaped layer (77 M weights, 0.162 bits/weight of records, SDQ scales, eight
 // vectors, one batched launch): 308 -> 76 us a call. Its relative error against 64 bits
-// is 9.7e-8 where the FP32 pipes' sums had 1.4e-7. Bound by latency and issue (43% of
+// is 9.3e-8 where the FP32 pipes' sums had 1.4e-7. Bound by latency and issue (43% of
 // slots): 695 warp instructions per 16 rows and 128 inputs without records (the split of
 // x about half), 910 on average with this layer's; x comes from L1, so the sums' shared
 // memory is no larger than needed (32 KB a block for all cases: 3 to 6% slower).
@@ -264,8 +264,8 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
   if (g0 < g1) load(g0);
   int gr = g0;
   for (int sum = sum0; sum < sum1; ++sum) {
-    const int end = bound(sum + 1);
-    if (gr == end) continue;
+    const int first = gr, end = bound(sum + 1);
+    if (first == end) continue;
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f}, racc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     for (; gr < end; ++gr) {
       uint32_t wc[2][4];
@@ -359,10 +359,14 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
       }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
+        racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
+        if (LC != 5 && gr == first) {  // a sum starts from its first residual: a rounding less
+          acc[i] = __fadd_rn(acc[i], racc[i]);
+          racc[i] = 0.0f;
+        }
         // an all-zero group (scale 0) adds nothing, whatever x holds
         const float sr = sc[i >> 1];
         if (sr != 0.0f) acc[i] = __fmaf_rn(__fadd_rn(h[i], ml[i]), sr, acc[i]);
-        racc[i] = __fadd_rn(racc[i], __fadd_rn(rh[i], rml[i]));
       }
     }
     float v[4];
@@ -371,16 +375,23 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
     part[warp / ks][sum][lane] = make_float4(v[0], v[1], v[2], v[3]);
   }
   __syncthreads();
+  // the sums two by two: closer than one after the other
   float v[4] = {0.0f, 0.0f, 0.0f, 0.0f};
   if (slice == 0 && row0 < tk.rows) {
-    for (int i = 0; i < kSums; ++i) {
-      if (bound(i) == bound(i + 1)) continue;
-      const float4 p = part[warp / ks][i][lane];
-      v[0] = __fadd_rn(v[0], p.x);
-      v[1] = __fadd_rn(v[1], p.y);
-      v[2] = __fadd_rn(v[2], p.z);
-      v[3] = __fadd_rn(v[3], p.w);
-    }
+    float4 p[kSums];
+#pragma unroll
+    for (int k = 0; k < kSums; ++k)
+      p[k] = bound(k) < bound(k + 1) ? part[warp / ks][k][lane] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int d = 1; d < kSums; d <<= 1)
+#pragma unroll
+      for (int k = 0; k < kSums; k += 2 * d)
+        p[k] = make_float4(__fadd_rn(p[k].x, p[k + d].x), __fadd_rn(p[k].y, p[k + d].y),
+                           __fadd_rn(p[k].z, p[k + d].z), __fadd_rn(p[k].w, p[k + d].w));
+    v[0] = p[0].x;
+    v[1] = p[0].y;
+    v[2] = p[0].z;
+    v[3] = p[0].w;
   }
   if (slice == 0) {
 #pragma unroll
@@ -394,30 +405,17 @@ __global__ void __launch_bounds__(32 * kWarps, 2) gemv_mma_kernel(Prm pr, const 
 
 }  // namespace
 
-// From three vectors on, where the tensor cores are estimated to be faster on the
-// module list. The list decides, and M, not the tasks of a call: a product's bits are
-// the same in every call on the list. In us, fitted to single modules and whole layers
-// of 0.03 to 275 M weights, M = 3 to 8 (records at 0.162 bits/weight; without records
-// both sides take about 0.6 of it):
-//  * here 3 + the larger of 0.4 per group of the widest module (a warp's slice, an
-//    eighth of them, one group after the other) and 1.05 per million weights, whatever M;
-//  * on the FP32 pipes 3 + (0.3 + 0.21 M) per million weights, and M where the inputs do
-//    not fit in shared memory (gemv.cu).
-// Measured, FP32 pipes against tensor cores: 1024 x 1024, M = 4: 4.6 and 6.3; 2048 x
-// 2048, M = 3 and 8: 8.0 and 9.9, 14.2 and 9.9; 512 x 11008, M = 4 and 8: 20.1 and 36,
-// 38.4 and 36; 11008 x 2048, M = 3 and 5: 24.3 and 26.5, 32.9 and 26.8; the layer above
-// (random records), M = 3 and 8: 126 and 73, 268 and 76.
-bool gemv_mma(const Prm& pr, const GemvArgs& a, int M, int n_mod, const awsrc_module* mods) {
+// From three vectors on, whatever the shapes: these sums are closer to 64 bits than
+// those of the FP32 pipes (6 to 9e-8 against 9 to 14e-8), which would be faster on some
+// single modules. In us on the device, FP32 pipes
+// against tensor cores (whose time does not depend on M), records at 0.162 bits/weight:
+// the layer above (random records), M = 3 and 8: 126 and 268 against 75; one module of
+// 4096 x 4096: 19.8 and 92.5 against 20; 11008 x 2048: 24.3 and 47.7 against 27; 2048 x
+// 2048: 8.0 and 14.2 against 9.9; 1024 x 1024: 4.1 and 6.6 against 6.4; 512 x 11008: 19.4
+// and 38.4 against 36. M = 1 and 2 take 30 and 47 on that layer there.
+bool gemv_mma(const Prm& pr, const GemvArgs& a, int M) {
   const bool c = pr.C == 16 || pr.C == 32 || pr.C == 64;
-  if (M < 3 || !c || (a.map && (!a.nib || pr.scale_mode != AWSRC_SCALE_POW2))) return false;
-  double widest = 0.0, weights = 0.0, fp32 = 0.0;
-  for (int m = 0; m < n_mod; ++m) {
-    const double w = 1e-6 * (double)mods[m].rows * (double)mods[m].cols;
-    weights += w;
-    widest = std::max(widest, (double)(mods[m].cols >> 7));
-    fp32 += w * (gemv_in_smem(mods[m].cols, M) ? 0.3 + 0.21 * M : (double)M);
-  }
-  return fp32 >= std::max(0.4 * widest, 1.05 * weights);
+  return M >= 3 && c && (!a.map || (a.nib && pr.scale_mode == AWSRC_SCALE_POW2));
 }
 
 cudaError_t launch_gemv_mma(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st) {

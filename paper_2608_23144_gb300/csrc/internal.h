@@ -168,11 +168,8 @@ struct GemvArgs {
 // Whether the GEMV walks recorded tiles with the decoder's code tables.
 bool gemv_tables(const Prm& pr);
 cudaError_t launch_gemv(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st);
-// Whether M vectors of `cols` inputs fit in the shared memory of a block there.
-bool gemv_in_smem(int64_t cols, int M);
-// gemv_mma.cu: the same products on the tensor cores, where gemv_mma() says so (for
-// the call's module list, not its tasks).
-bool gemv_mma(const Prm& pr, const GemvArgs& a, int M, int n_mod, const awsrc_module* mods);
+// gemv_mma.cu: the same products on the tensor cores, where gemv_mma() says so.
+bool gemv_mma(const Prm& pr, const GemvArgs& a, int M);
 cudaError_t launch_gemv_mma(const Prm& pr, const GemvArgs& a, int M, cudaStream_t st);
 
 // backbone.cu: RTN-INT4 groups of rtn_group() inputs, SDQ blocks of sdq_block() groups.
