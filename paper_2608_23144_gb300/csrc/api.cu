@@ -530,9 +530,11 @@ awsrc_status awsrc_encode_tiles(const awsrc_params* prm, int32_t n_mod, const aw
     if (lay.nsplit > 1) {  // best of the seed splits of each tile
       const int64_t t0 = ld.m[0].tile_off;
       const int64_t t1 = ld.m[ld.n - 1].tile_off + ld.m[ld.n - 1].rows * ld.m[ld.n - 1].n_cb;
-      // early behind a search of one wave (1.3 us less at 512 tiles and 256 seeds); behind
-      // more, the blocks that wait only disturb it (512 x 512, C = 64, S = 1024: 117 -> 125 us)
-      const bool early = blocks <= (lay.mma ? search_mma_slots(pr) : kSms);
+      // early behind a search of one wave (1.3 us less at 512 tiles and 256 seeds) or one
+      // that lets nothing start before it ends (P_F with C = 64, P = 4, the scalar one: the
+      // launch alone is 4 us of 205); behind several waves of the others the blocks that
+      // wait only disturb it (512 x 512, C = 64, S = 1024: 117 -> 125 us)
+      const bool early = !(lay.spec || lay.mma) || blocks <= (lay.mma ? search_mma_slots(pr) : kSms);
       if ((e = launch_merge_candidates(pcands, lay.nsplit, T, t0, t1, early, out, st)) != cudaSuccess)
         return cuda_fail(e, "encode: merge");
     }
