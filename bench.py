@@ -59,8 +59,8 @@ def search_algorithmic_bytes(weights: int, tiles: int) -> int:
     return 4 * weights + 16 * tiles
 # DRAM traffic (read + write) of one full-layer search launch, from an ncu launch
 # list of this workload; valid only for the kernel source it was measured on.
-SEARCH_TRAFFIC = {"source_sha256": "83323cd64dc70a1b688b0fbb25a68c21e6b8daaf0d4bbe37da28cfa6932d3a77",
-                  "bytes_per_launch": 443149056 + 18763776,
+SEARCH_TRAFFIC = {"source_sha256": "b6fbca151a967311985d4c74cada4f870255f2355a5b9ce51b25bd8037029d7f",
+                  "bytes_per_launch": 443387392 + 18991104,
                   # the same kernel's pipe utilisation in an ncu capture (gate + up)
                   "ncu_fma_pipe_pct": 40.20, "ncu_issue_active_pct": 48.47,
                   "ncu_tensor_pipe_pct": 24.67}
